@@ -382,6 +382,7 @@ void apply_tiling(sc_lbm_t h) {
     D.tiles_per_node = D.tiles_x * D.tiles_y * D.tiles_z;
     D.tile_begin = begin;
     begin += D.tiles_per_node * D.nodes;
+    set_tile_divisions(D, P.order);
     D.bitem_begin = bbegin;
     bbegin += D.nb * D.nodes;
     D.runs_per_node = D.pitch / kRun;

@@ -547,6 +547,7 @@ void hn_link_words(const sc_domain_desc& D, const uint8_t* flags, std::vector<Li
             }
           }
           word |= (LinkWord)kind << (2 * i);
+          if (kind == kSpecZ) word |= kLinkSpec;
         }
         if (complex_cell) word |= kLinkComplex;
         if (vel) word |= kLinkVel;

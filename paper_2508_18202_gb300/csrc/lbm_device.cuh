@@ -156,60 +156,118 @@ __device__ __forceinline__ uint16_t ld_keep(const uint16_t* p) {
 __device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
 __device__ __forceinline__ double recip(double x) { return __drcp_rn(x); }
 
+// c_i . u for a direction known at compile time: only the components the
+// direction has.  Written as T(CX(i)) * ux + ..., IEEE arithmetic has the
+// compiler keep the products by zero (0 * u is not 0 for every u), two
+// instructions of three on the axis directions and one on the diagonals; for
+// finite u the sum has the same bits.
+// The unit of the regularized collision keeps the full products, and sums
+// that start from 0: which of that collision's products the compiler fuses
+// into additions follows from the code around them, and this form leaves its
+// results as they are.
+template <class T>
+__device__ __forceinline__ T cdot(int i, T ux, T uy, T uz) {
+#ifdef SCLBM_RR_UNIT
+  return T(CX(i)) * ux + T(CY(i)) * uy + T(CZ(i)) * uz;
+#endif
+  T s = T(0);
+  if (CX(i)) s = CX(i) > 0 ? ux : -ux;
+  if (CY(i)) s = CX(i) ? (CY(i) > 0 ? s + uy : s - uy) : (CY(i) > 0 ? uy : -uy);
+  if (CZ(i)) s = (CX(i) || CY(i)) ? (CZ(i) > 0 ? s + uz : s - uz) : (CZ(i) > 0 ? uz : -uz);
+  return s;
+}
+
+// sum_i g_i and sum_i c_i g_i in ascending order of i; each sum starts from
+// its first term (a start from 0 is one more addition).
+template <class T>
+__device__ __forceinline__ void flow_sums(const T g[kQ], T& m0, T& jx, T& jy, T& jz) {
+  m0 = g[0], jx = g[1], jy = g[3], jz = g[5];
+#pragma unroll
+  for (int i = 1; i < kQ; ++i) {
+    m0 += g[i];
+    if (CX(i) && i > 1) jx += CX(i) > 0 ? g[i] : -g[i];
+    if (CY(i) && i > 3) jy += CY(i) > 0 ? g[i] : -g[i];
+    if (CZ(i) && i > 5) jz += CZ(i) > 0 ? g[i] : -g[i];
+  }
+}
+// The same with the second moments sum_i c_i c_i g_i.
+template <class T>
+__device__ __forceinline__ void all_sums(const T g[kQ], T& m0, T& jx, T& jy, T& jz, T& pxx, T& pyy, T& pzz, T& pxy,
+                                         T& pxz, T& pyz) {
+#ifdef SCLBM_RR_UNIT
+  constexpr int kFirst = -1;
+  m0 = jx = jy = jz = pxx = pyy = pzz = pxy = pxz = pyz = T(0);
+#else
+  constexpr int kFirst = 0;  // the terms taken as the starting values: i = 0, and the first of each sum
+  m0 = g[0], jx = g[1], jy = g[3], jz = g[5];
+  pxx = g[1], pyy = g[3], pzz = g[5], pxy = g[7], pxz = g[11], pyz = g[15];
+#endif
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) {
+    if (i > kFirst) m0 += g[i];
+    if (CX(i) && (kFirst < 0 || i > 1)) jx += CX(i) > 0 ? g[i] : -g[i];
+    if (CY(i) && (kFirst < 0 || i > 3)) jy += CY(i) > 0 ? g[i] : -g[i];
+    if (CZ(i) && (kFirst < 0 || i > 5)) jz += CZ(i) > 0 ? g[i] : -g[i];
+    if (CX(i) && (kFirst < 0 || i > 1)) pxx += g[i];
+    if (CY(i) && (kFirst < 0 || i > 3)) pyy += g[i];
+    if (CZ(i) && (kFirst < 0 || i > 5)) pzz += g[i];
+    if (CX(i) * CY(i) && (kFirst < 0 || i > 7)) pxy += CX(i) * CY(i) > 0 ? g[i] : -g[i];
+    if (CX(i) * CZ(i) && (kFirst < 0 || i > 11)) pxz += CX(i) * CZ(i) > 0 ? g[i] : -g[i];
+    if (CY(i) * CZ(i) && (kFirst < 0 || i > 15)) pyz += CY(i) * CZ(i) > 0 ? g[i] : -g[i];
+  }
+}
+
+// Single operations, each rounded once: the collision below fixes which
+// products are fused into additions, so every kernel that carries it (each
+// level, launch shape, precision of storage and execution mode, and the
+// adjoint's forward) gives the same bits however the compiler schedules it.
+__device__ __forceinline__ float mul1(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul1(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float add1(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add1(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float fma1(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma1(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // BGK with the Smagorinsky effective relaxation time (Sec. 2.2).  SHIFT:
 // populations are g = f - w.  The non-equilibrium stress uses the exact
 // second moment of the D3Q19 second-order equilibrium, rho/3 I + rho u u.
 template <class T, bool SHIFT>
 __device__ __forceinline__ void collide(T g[kQ], T tau0, T smag18c2, bool smag_on) {
-  T m0 = T(0), jx = T(0), jy = T(0), jz = T(0);
-  T pxx = T(0), pyy = T(0), pzz = T(0), pxy = T(0), pxz = T(0), pyz = T(0);
-#pragma unroll
-  for (int i = 0; i < kQ; ++i) {
-    m0 += g[i];
-    if (CX(i)) jx += CX(i) > 0 ? g[i] : -g[i];
-    if (CY(i)) jy += CY(i) > 0 ? g[i] : -g[i];
-    if (CZ(i)) jz += CZ(i) > 0 ? g[i] : -g[i];
-    if (CX(i)) pxx += g[i];
-    if (CY(i)) pyy += g[i];
-    if (CZ(i)) pzz += g[i];
-    if (CX(i) * CY(i)) pxy += CX(i) * CY(i) > 0 ? g[i] : -g[i];
-    if (CX(i) * CZ(i)) pxz += CX(i) * CZ(i) > 0 ? g[i] : -g[i];
-    if (CY(i) * CZ(i)) pyz += CY(i) * CZ(i) > 0 ? g[i] : -g[i];
-  }
-  const T rho = SHIFT ? T(1) + m0 : m0;
+  T m0, jx, jy, jz, pxx, pyy, pzz, pxy, pxz, pyz;
+  all_sums<T>(g, m0, jx, jy, jz, pxx, pyy, pzz, pxy, pxz, pyz);
+  const T rho = SHIFT ? add1(T(1), m0) : m0;
   const T inv = recip(rho);
-  const T ux = jx * inv, uy = jy * inv, uz = jz * inv;
-  const T usq = ux * ux + uy * uy + uz * uz;
+  const T ux = mul1(jx, inv), uy = mul1(jy, inv), uz = mul1(jz, inv);
+  const T usq = fma1(uz, uz, fma1(ux, ux, mul1(uy, uy)));
   T tau = tau0;
   if (smag_on) {
     // Pi^neq = sum c c g - (m0/3 I + rho u u); m0 = rho - 1 (shifted) or rho
-    const T third = m0 * T(1.0 / 3.0);
-    const T nxx = pxx - third - rho * ux * ux;
-    const T nyy = pyy - third - rho * uy * uy;
-    const T nzz = pzz - third - rho * uz * uz;
-    const T nxy = pxy - rho * ux * uy;
-    const T nxz = pxz - rho * ux * uz;
-    const T nyz = pyz - rho * uy * uz;
-    const T pipi = nxx * nxx + nyy * nyy + nzz * nzz + T(2) * (nxy * nxy + nxz * nxz + nyz * nyz);
-    const T pin = sqrt(T(2) * pipi + T(1e-30));
-    tau = T(0.5) * (tau0 + sqrt(tau0 * tau0 + smag18c2 * pin * inv));
+    const T rx = mul1(rho, ux), ry = mul1(rho, uy), rz = mul1(rho, uz);
+    const T nxx = fma1(-rx, ux, fma1(-m0, T(1.0 / 3.0), pxx));
+    const T nyy = fma1(-ry, uy, fma1(-m0, T(1.0 / 3.0), pyy));
+    const T nzz = fma1(-rz, uz, fma1(-m0, T(1.0 / 3.0), pzz));
+    const T nxy = fma1(-rx, uy, pxy);
+    const T nxz = fma1(-rx, uz, pxz);
+    const T nyz = fma1(-ry, uz, pyz);
+    const T dia = fma1(nzz, nzz, fma1(nxx, nxx, mul1(nyy, nyy)));
+    const T off = fma1(nyz, nyz, fma1(nxy, nxy, mul1(nxz, nxz)));
+    const T pin = sqrt(fma1(T(2), fma1(T(2), off, dia), T(1e-30)));
+    tau = mul1(T(0.5), add1(tau0, sqrt(fma1(tau0, tau0, mul1(mul1(smag18c2, pin), inv)))));
   }
   const T omega = recip(tau);
-  const T base = m0;  // shifted: w (rho - 1) part; plain: w rho part
   // Opposite pairs (i, i + 1), i odd, share c_i . u up to the sign: the
   // bracket of the equilibrium splits into an even part
-  // base + rho (4.5 cu^2 - 1.5 u^2) and an odd part 3 rho cu; the weight
-  // multiplies last (a rounded 3 w would bias the momentum of every
-  // collision).
-  const T r15 = T(1.5) * usq;
-  g[0] = g[0] - omega * (g[0] - W<T>(0) * (base - rho * r15));
+  // m0 + rho (4.5 cu^2 - 1.5 u^2) (m0: w (rho - 1) shifted, w rho plain) and
+  // an odd part 3 rho cu; the weight multiplies last (a rounded 3 w would
+  // bias the momentum of every collision).
+  const T r15 = mul1(T(1.5), usq), r3 = mul1(T(3), rho);
+  g[0] = fma1(-omega, fma1(-W<T>(0), fma1(-rho, r15, m0), g[0]), g[0]);
 #pragma unroll
   for (int i = 1; i < kQ; i += 2) {
-    const T cu = T(CX(i)) * ux + T(CY(i)) * uy + T(CZ(i)) * uz;
-    const T even = base + rho * (T(4.5) * cu * cu - r15);
-    const T odd = T(3) * rho * cu;
-    g[i] = g[i] - omega * (g[i] - W<T>(i) * (even + odd));
-    g[i + 1] = g[i + 1] - omega * (g[i + 1] - W<T>(i) * (even - odd));
+    const T cu = cdot<T>(i, ux, uy, uz);
+    const T even = fma1(rho, fma1(mul1(T(4.5), cu), cu, -r15), m0);
+    g[i] = fma1(-omega, fma1(-W<T>(i), fma1(r3, cu, even), g[i]), g[i]);
+    g[i + 1] = fma1(-omega, fma1(-W<T>(i), fma1(-r3, cu, even), g[i + 1]), g[i + 1]);
   }
 }
 
@@ -244,21 +302,8 @@ __host__ __device__ constexpr double H3K(int i, int k) {
 // in collide (the rho part then carries rho - 1).
 template <class T, bool SHIFT>
 __device__ __forceinline__ void collide_rr(T g[kQ], T tau0, T smag18c2, bool smag_on) {
-  T m0 = T(0), jx = T(0), jy = T(0), jz = T(0);
-  T pxx = T(0), pyy = T(0), pzz = T(0), pxy = T(0), pxz = T(0), pyz = T(0);
-#pragma unroll
-  for (int i = 0; i < kQ; ++i) {
-    m0 += g[i];
-    if (CX(i)) jx += CX(i) > 0 ? g[i] : -g[i];
-    if (CY(i)) jy += CY(i) > 0 ? g[i] : -g[i];
-    if (CZ(i)) jz += CZ(i) > 0 ? g[i] : -g[i];
-    if (CX(i)) pxx += g[i];
-    if (CY(i)) pyy += g[i];
-    if (CZ(i)) pzz += g[i];
-    if (CX(i) * CY(i)) pxy += CX(i) * CY(i) > 0 ? g[i] : -g[i];
-    if (CX(i) * CZ(i)) pxz += CX(i) * CZ(i) > 0 ? g[i] : -g[i];
-    if (CY(i) * CZ(i)) pyz += CY(i) * CZ(i) > 0 ? g[i] : -g[i];
-  }
+  T m0, jx, jy, jz, pxx, pyy, pzz, pxy, pxz, pyz;
+  all_sums<T>(g, m0, jx, jy, jz, pxx, pyy, pzz, pxy, pxz, pyz);
   const T rho = SHIFT ? T(1) + m0 : m0;
   const T inv = recip(rho);
   const T ux = jx * inv, uy = jy * inv, uz = jz * inv;
@@ -292,7 +337,7 @@ __device__ __forceinline__ void collide_rr(T g[kQ], T tau0, T smag18c2, bool sma
   const T base = m0;
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
-    const T cu = T(CX(i)) * ux + T(CY(i)) * uy + T(CZ(i)) * uz;
+    const T cu = cdot<T>(i, ux, uy, uz);
     T v = base + rho * (T(3) * cu + T(4.5) * cu * cu - T(1.5) * usq);
     v += T(CX(i) * CX(i) - 1.0 / 3.0) * kxx + T(CY(i) * CY(i) - 1.0 / 3.0) * kyy +
          T(CZ(i) * CZ(i) - 1.0 / 3.0) * kzz;
@@ -475,7 +520,7 @@ struct Node {
 // velocity turned to the arrival level's direction, r its scale.
 template <class T>
 __device__ __forceinline__ T wall_term(int i, T ux, T uy, T uz, T r) {
-  return T(6) * W<T>(i) * (T(CX(i)) * ux + T(CY(i)) * uy + T(CZ(i)) * uz) * r;
+  return T(6) * W<T>(i) * cdot<T>(i, ux, uy, uz) * r;
 }
 
 // Pull of the odd AA level (swapped layout in place).
@@ -514,6 +559,76 @@ __device__ __forceinline__ void fast_push(S* base, LinkWord lw, int pc, int sy, 
     T v = g[j];
     if (kind == kMoving) v += wall_term<T>(OPP(j), ux, uy, uz, r1);
     Store<S>::st(base + off, v);
+  }
+}
+
+// Whether link i can be of kind kSpecZ with a slot of its own: it crosses a z
+// face (on the pure z directions the in-plane neighbour is the cell itself,
+// and the specular slot is the bounce-back one).
+__host__ __device__ constexpr bool SPECZ(int i) { return CZ(i) != 0 && (CX(i) != 0 || CY(i) != 0); }
+
+// The kinds of a link word as masks, one bit per link at bit 2i of a 64-bit
+// word (kept as two 32-bit halves): links that do not stream, moving-wall
+// links, specular links.
+struct LinkMasks {
+  uint32_t wall[2], move[2], spec[2];
+  __device__ __forceinline__ explicit LinkMasks(LinkWord lw) {
+    const uint32_t w[2] = {(uint32_t)lw, (uint32_t)((lw & kLinkKinds) >> 32)};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint32_t hi = w[h] >> 1;
+      wall[h] = w[h] | hi;
+      move[h] = hi & ~w[h];
+      spec[h] = hi & w[h];
+    }
+  }
+  static __device__ __forceinline__ int bit(const uint32_t m[2], int i) {
+    return (int)((m[i >> 4] >> (2 * (i & 15))) & 1u);
+  }
+};
+
+// The same rules for the bulk cells of the in-place odd level.  GENERAL: a
+// cell of the warp has a moving-wall or specular link; without it every link
+// streams or bounces back.  A link's address is selected by one multiply-add
+// of its "does not stream" bit: two instructions a link instead of the
+// comparisons, selects and predicated wall term of the forms above, which
+// cost the warps that touch a building or the ground about as much again as
+// their collision.
+template <class S, bool CG, bool GENERAL>
+__device__ __forceinline__ void mask_pull(const S* base, LinkWord lw, int pc, int sy, int sz,
+                                          typename Store<S>::C ux, typename Store<S>::C uy,
+                                          typename Store<S>::C uz, typename Store<S>::C r,
+                                          typename Store<S>::C g[kQ]) {
+  using T = typename Store<S>::C;
+  const LinkMasks m(lw);
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) {
+    const int stream = OPP(i) * pc - (CX(i) + CY(i) * sy + CZ(i) * sz);
+    int off = stream + LinkMasks::bit(m.wall, i) * (i * pc - stream);
+    if (GENERAL && SPECZ(i))
+      off += LinkMasks::bit(m.spec, i) * (OPP(REFL(i, 2)) * pc - (CX(i) + CY(i) * sy) - i * pc);
+    T v = LD<S, CG>(base + (i == 0 ? 0 : off));
+    if (GENERAL && i > 0 && LinkMasks::bit(m.move, i)) v += wall_term<T>(i, ux, uy, uz, r);
+    g[i] = v;
+  }
+}
+
+template <class S, bool GENERAL>
+__device__ __forceinline__ void mask_push(S* base, LinkWord lw, int pc, int sy, int sz,
+                                          typename Store<S>::C ux, typename Store<S>::C uy,
+                                          typename Store<S>::C uz, typename Store<S>::C r1,
+                                          const typename Store<S>::C g[kQ]) {
+  using T = typename Store<S>::C;
+  const LinkMasks m(lw);
+#pragma unroll
+  for (int j = 0; j < kQ; ++j) {
+    const int stream = j * pc + (CX(j) + CY(j) * sy + CZ(j) * sz);
+    int off = stream + LinkMasks::bit(m.wall, OPP(j)) * (OPP(j) * pc - stream);
+    if (GENERAL && SPECZ(j))
+      off += LinkMasks::bit(m.spec, OPP(j)) * (REFL(j, 2) * pc + (CX(j) + CY(j) * sy) - OPP(j) * pc);
+    T v = g[j];
+    if (GENERAL && j > 0 && LinkMasks::bit(m.move, OPP(j))) v += wall_term<T>(OPP(j), ux, uy, uz, r1);
+    Store<S>::st(base + (j == 0 ? 0 : off), v);
   }
 }
 

@@ -86,13 +86,49 @@ __device__ __forceinline__ void cell_even(const StepParams& P, const DevDomain& 
 
 // ------------------------------------------------------------ step driver
 // A tile is a block_x * block_y patch of one x-y plane range, slab_z deep,
-// of one node of one domain.  Decoded once per block (32-bit arithmetic; tile
-// counts stay below 2^31) and shared with the block's threads.
+// of one node of one domain.
 struct TileRef {
   int d, node, x, y, z0, z1;
   bool valid;
 };
 
+__device__ __forceinline__ unsigned fdiv(unsigned n, const FastDiv& f) {
+  return f.m ? __umulhi(n, f.m) >> f.shift : n;
+}
+
+// The step kernels of the BGK collision: every thread decodes the tile index
+// with 32-bit reciprocal multiplications (tile counts stay below 2^31).  The
+// index comes from blockIdx alone, so the decode, the domain's fields and the
+// strides that follow from them can stay in uniform registers, and the block
+// needs no shared-memory broadcast and no barrier before its first loads.
+// CPT: x-adjacent cells per thread (the tile is then CPT * blockDim.x cells
+// wide, P.bx = CPT * blockDim.x); R.x is the thread's first cell.
+#ifndef SCLBM_RR_UNIT
+template <int CPT = 1>
+__device__ __forceinline__ TileRef block_tile(const StepParams& P, unsigned t) {
+  int d = 0;
+  for (int k = 1; k < P.n_domains; ++k)
+    if (t >= (unsigned)P.dom[k].tile_begin) d = k;
+  const DevDomain& D = P.dom[d];
+  const unsigned local = t - (unsigned)D.tile_begin;
+  const unsigned q = fdiv(local, D.by_major);
+  const unsigned rest = local - q * (P.order == 0 ? (unsigned)D.nodes : (unsigned)D.tiles_per_node);
+  const unsigned node = P.order == 0 ? rest : q, ct = P.order == 0 ? q : rest;
+  const unsigned tx = (unsigned)D.tiles_x, txy = tx * (unsigned)D.tiles_y;
+  const unsigned tz = fdiv(ct, D.by_txy), rem = ct - tz * txy;
+  const unsigned ty = fdiv(rem, D.by_tx);
+  TileRef R;
+  R.d = d;
+  R.node = (int)node;
+  R.x = (int)(rem - ty * tx) * P.bx + CPT * threadIdx.x;
+  R.y = (int)ty * P.by + threadIdx.y;
+  R.z0 = (int)tz * P.bz;
+  R.z1 = min(R.z0 + P.bz, D.nz);
+  R.valid = R.x < D.nx && R.y < D.ny;
+  return R;
+}
+#else
+// The regularized collision's kernels: decoded once per block and shared.
 struct TileHead {
   int d, node, x0, y0, z0;
 };
@@ -143,6 +179,7 @@ __device__ __forceinline__ TileRef block_tile(const StepParams& P, unsigned t) {
   R.valid = R.x < D.nx && R.y < D.ny;
   return R;
 }
+#endif
 
 // Even level over the z-slab of a tile.  The link word of the next cell is
 // loaded one cell ahead so the population loads do not wait on it.
@@ -161,11 +198,22 @@ __device__ __forceinline__ void even_run(const StepParams& P, S* base, const uin
     if (k + 1 < n) next = ld_keep(cp + plane);
     if (cls & kClsSkip) continue;
     T g[kQ];
+#ifndef SCLBM_RR_UNIT
+    // the 19 row offsets are loop-invariant: hidden from the optimiser per
+    // cell they are one multiply-add each instead of spilled registers
+    int pcv = pc;
+    asm volatile("" : "+r"(pcv));
+#else
+    const int pcv = pc;
+#endif
 #pragma unroll
-    for (int i = 0; i < kQ; ++i) g[i] = LD<S, CG>(base + i * pc);
+    for (int i = 0; i < kQ; ++i) g[i] = LD<S, CG>(base + i * pcv);
     collide_p<T, true>(P, g);
+#ifndef SCLBM_RR_UNIT
+    asm volatile("" : "+r"(pcv));
+#endif
 #pragma unroll
-    for (int i = 0; i < kQ; ++i) Store<S>::st(base + OPP(i) * pc, g[i]);
+    for (int i = 0; i < kQ; ++i) Store<S>::st(base + OPP(i) * pcv, g[i]);
   }
 }
 
@@ -193,7 +241,7 @@ __device__ __forceinline__ void even_tile(const StepParams& P, const TileRef& R)
 
 // Odd level over the z-slab of a tile.  A warp whose cells are all interior
 // (or skipped) takes the plain streaming form; a warp with any wall, inflow
-// or lid link takes the link-kind form for all its cells, so neither
+// or lid link takes a form with link kinds for all its cells, so none
 // diverges.  The next cell's link word is loaded one cell ahead.
 // ROT: the launch's factors may turn the inflow (a series); without it the
 // table velocity is read once and only scaled, which keeps the 64-register
@@ -215,6 +263,52 @@ __device__ __forceinline__ void odd_bulk_tile(const StepParams& P, const TileRef
   for (int z = R.z0; z < R.z1; ++z, base += sz, lp += sz) {
     const LinkWord lw = next;
     if (z + 1 < R.z1) next = ld_keep(lp + sz);
+#ifndef SCLBM_RR_UNIT
+    // the form of the warp's links: all stream; some bounce back; some are
+    // moving walls or specular.  One collision between the pulls and the
+    // pushes of the three (a collision in each holds more registers than the
+    // 64 of the 4-block kernels: 88 bytes spilled, odd level 779 us against
+    // 717 on the 13-sample 256 x 128 x 64 ensemble).
+    const unsigned active = __activemask();
+    const bool skip = (lw & kLinkSlow) != 0;   // solid, outlet or general-boundary cell
+    const bool interior = __all_sync(active, lw == 0 || skip);
+    T g[kQ];
+    // The 19 neighbour offsets are loop-invariant; hoisted out of the z
+    // loop they would hold 19 registers and spill at the 64-register
+    // budget.  Hiding the strides from the optimiser per cell makes each
+    // offset one multiply-add at its load or store instead.
+    int pcv = pc, syv = sy, szv = sz;
+    const bool general = __any_sync(active, !skip && (lw & kLinkGeneral));
+    if (skip) continue;
+    T ux, uy, uz;
+    Node<S> N;
+    N.g = nullptr;
+    N.bout = nullptr;
+    N.uinf = uinf;
+    N.uind = uind;
+    asm volatile("" : "+r"(pcv), "+r"(syv), "+r"(szv));
+    if (interior) {
+#pragma unroll
+      for (int i = 0; i < kQ; ++i)
+        g[i] = LD<S, CG>(base + (OPP(i) * pcv - (CX(i) + CY(i) * syv + CZ(i) * szv)));
+    } else if (!general) {
+      mask_pull<S, CG, false>(base, lw, pcv, syv, szv, T(0), T(0), T(0), T(0), g);
+    } else {
+      wall_velocity<S, ROT>(N, lw, z, wind_pull<T>(P), ux, uy, uz);
+      mask_pull<S, CG, true>(base, lw, pcv, syv, szv, ux, uy, uz, wind_pull<T>(P).scale, g);
+    }
+    collide_p<T, true>(P, g);
+    asm volatile("" : "+r"(pcv), "+r"(syv), "+r"(szv));
+    if (interior) {
+#pragma unroll
+      for (int j = 0; j < kQ; ++j) Store<S>::st(base + (j * pcv + (CX(j) + CY(j) * syv + CZ(j) * szv)), g[j]);
+    } else if (!general) {
+      mask_push<S, false>(base, lw, pcv, syv, szv, T(0), T(0), T(0), T(0), g);
+    } else {
+      wall_velocity<S, ROT>(N, lw, z, wind_push<T>(P), ux, uy, uz);
+      mask_push<S, true>(base, lw, pcv, syv, szv, ux, uy, uz, wind_push<T>(P).scale, g);
+    }
+#else
     const bool interior = __all_sync(__activemask(), lw == 0 || (lw & kLinkSlow));
     if (lw & kLinkSlow) continue;   // solid, outlet or general-boundary cell
     T g[kQ];
@@ -245,6 +339,7 @@ __device__ __forceinline__ void odd_bulk_tile(const StepParams& P, const TileRef
       if constexpr (ROT) wall_velocity<S>(N, lw, z, wind_push<T>(P), ux, uy, uz);
       fast_push<S>(base, lw, pc, sy, sz, ux, uy, uz, wind_push<T>(P).scale, g);
     }
+#endif
   }
 }
 
@@ -309,19 +404,18 @@ __device__ __forceinline__ void even_boundary_item(const StepParams& P, long lon
 // launch.  Returns true for a listed block, with its rank among the listed
 // blocks in *index, else the rank among the bulk blocks (the tile index).
 __device__ __forceinline__ bool block_role(const StepParams& P, unsigned* index) {
-  const long long threads = (long long)blockDim.x * blockDim.y;
-  const unsigned listed = (unsigned)((P.total_bitems + threads - 1) / threads);
   const unsigned b = blockIdx.x;
-  if (listed == 0) {
+  if (P.listed_blocks == 0) {
     *index = b;
     return false;
   }
-  const unsigned q = gridDim.x / listed;  // >= 1: the grid is tiles + listed blocks
-  if (b % q == 0 && b / q < listed) {
-    *index = b / q;
+  const unsigned rank = fdiv(b, P.by_listed_every);
+  const bool on = b == rank * P.listed_every;
+  if (on && rank < P.listed_blocks) {
+    *index = rank;
     return true;
   }
-  *index = b - min((b + q - 1) / q, listed);
+  *index = b - min(on ? rank : rank + 1, P.listed_blocks);
   return false;
 }
 
@@ -767,12 +861,16 @@ __global__ void __launch_bounds__(256, 3) aa_persistent_kernel(const __grid_cons
     if ((n & 1ull) == 0) {
       for (long long t = blockIdx.x; t < P.total_tiles; t += gridDim.x) {
         even_tile<S, true, false>(P, block_tile(P, (unsigned)t));
+#ifdef SCLBM_RR_UNIT
         __syncthreads();  // the shared tile head is rewritten next iteration
+#endif
       }
     } else {
       for (long long t = blockIdx.x; t < P.total_tiles; t += gridDim.x) {
         odd_bulk_tile<S, true, ROT>(P, block_tile(P, (unsigned)t));
+#ifdef SCLBM_RR_UNIT
         __syncthreads();
+#endif
       }
       // bulk and boundary cells touch disjoint slots: no barrier between them
       for (long long b = blockIdx.x; b < bblocks; b += gridDim.x)
@@ -905,11 +1003,23 @@ StepParams pair_tiling(const StepParams& P) {
     D.tiles_per_node = D.tiles_x * D.tiles_y * D.tiles_z;
     D.tile_begin = begin;
     begin += D.tiles_per_node * D.nodes;
+    set_tile_divisions(D, Q.order);
   }
   Q.total_tiles = begin;
   return Q;
 }
 #endif
+
+// The launch with its listed items in blocks of `threads` threads spread over
+// the grid of total_tiles bulk blocks; *grid receives the block count.
+StepParams with_listed_blocks(const StepParams& P, long long threads, unsigned* grid) {
+  StepParams Q = P;
+  Q.listed_blocks = (unsigned)((P.total_bitems + threads - 1) / threads);
+  *grid = (unsigned)(P.total_tiles + Q.listed_blocks);
+  Q.listed_every = Q.listed_blocks ? *grid / Q.listed_blocks : 1u;  // >= 1
+  Q.by_listed_every = fast_div(Q.listed_every);
+  return Q;
+}
 
 int launch_aa_step(const StepParams& P, int precision, void* stream, int parity) {
   dim3 block(P.bx, P.by);
@@ -926,13 +1036,14 @@ int launch_aa_step(const StepParams& P, int precision, void* stream, int parity)
       }
       // listed items ride in blocks spread over the per-thread launches
       const long long threads = (long long)P.bx * P.by;
-      const unsigned lgrid = (unsigned)(P.total_tiles + (P.total_bitems + threads - 1) / threads);
+      unsigned lgrid = 0;
+      const StepParams L = with_listed_blocks(P, threads, &lgrid);
       if (parity == 0) {
 #ifndef SCLBM_RR_UNIT
         if constexpr (sizeof(S) == 2) {
           if (P.even_pair && !P.tma) {
-            const StepParams Q = pair_tiling(P);
-            const unsigned qgrid = (unsigned)(Q.total_tiles + (Q.total_bitems + threads - 1) / threads);
+            unsigned qgrid = 0;
+            const StepParams Q = with_listed_blocks(pair_tiling(P), threads, &qgrid);
             if (P.even_pair == 3) aa_even_pair_kernel<S, 3><<<qgrid, block, 0, s>>>(Q);
             else aa_even_pair_kernel<S, 2><<<qgrid, block, 0, s>>>(Q);
             return (int)cudaGetLastError();
@@ -940,17 +1051,17 @@ int launch_aa_step(const StepParams& P, int precision, void* stream, int parity)
         }
 #endif
         if (P.tma) aa_even_tma_kernel<S><<<tgrid, kTmaThreads, even_tma_smem<S>(), s>>>(P);
-        else if (P.even85) aa_even_kernel<S, 3><<<lgrid, block, 0, s>>>(P);
-        else aa_even_kernel<S, 4><<<lgrid, block, 0, s>>>(P);
+        else if (P.even85) aa_even_kernel<S, 3><<<lgrid, block, 0, s>>>(L);
+        else aa_even_kernel<S, 4><<<lgrid, block, 0, s>>>(L);
       } else {
         if (P.tma) {
           aa_odd_tma_kernel<S><<<tgrid, kTmaThreads, odd_tma_smem<S>(), s>>>(P);
           const long long grid = (P.total_bitems + 255) / 256;
           aa_odd_boundary_kernel<S><<<(unsigned)(grid > 0 ? grid : 1), 256, 0, s>>>(P);
         } else if (P.odd85 || turns_inflow(P)) {
-          aa_odd_bulk_kernel<S, 3><<<lgrid, block, 0, s>>>(P);
+          aa_odd_bulk_kernel<S, 3><<<lgrid, block, 0, s>>>(L);
         } else {
-          aa_odd_bulk_kernel<S, 4><<<lgrid, block, 0, s>>>(P);
+          aa_odd_bulk_kernel<S, 4><<<lgrid, block, 0, s>>>(L);
         }
       }
       return (int)cudaGetLastError();

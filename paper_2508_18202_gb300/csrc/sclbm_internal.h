@@ -42,7 +42,10 @@ constexpr LinkWord kLinkSolid = 1ull << 40;    // the cell itself is solid
 constexpr LinkWord kLinkOutlet = 1ull << 41;   // fluid cell on an OUTFLOW +x face
 constexpr LinkWord kLinkComplex = 1ull << 42;  // some link needs the general rules
 constexpr LinkWord kLinkVel = 1ull << 43;      // some link carries the moving-wall term
+constexpr LinkWord kLinkSpec = 1ull << 44;     // some link is specular (kSpecZ)
 constexpr LinkWord kLinkKinds = (1ull << 38) - 1ull;
+// Cells of the fast path with links other than streaming and bounce-back.
+constexpr LinkWord kLinkGeneral = kLinkVel | kLinkSpec;
 // Cells without these bits take the fast path.
 constexpr LinkWord kLinkSlow = kLinkSolid | kLinkOutlet | kLinkComplex;
 
@@ -103,6 +106,23 @@ struct Wind {
 // beyond the mantle of a circular domain (links into it take the velocity rule).
 constexpr uint8_t kFlagMantle = 2;
 
+// Division of 0 <= n < 2^31 by a fixed d >= 1 as a multiplication by a rounded-up
+// reciprocal (Granlund & Montgomery, "Division by invariant integers using
+// multiplication", PLDI 1994): with 2^l >= d and m = floor(2^(31+l) / d) + 1 < 2^32
+// the quotient is the high part of n m, exactly.
+struct FastDiv {
+  uint32_t m, shift;  // n / d = (n * m) >> (31 + l), as (umulhi(n, m) >> shift) with shift = l - 1, or n for d = 1
+};
+inline FastDiv fast_div(uint32_t d) {
+  FastDiv f{0u, 0u};
+  if (d <= 1) return f;
+  uint32_t l = 0;
+  while ((1ull << l) < d) ++l;
+  f.m = (uint32_t)(((1ull << (31 + l)) / d) + 1ull);
+  f.shift = l - 1;
+  return f;
+}
+
 // Per-domain view handed to the kernels (plain pointers into the workspace).
 struct DevDomain {
   int nx, ny, nz, nodes;
@@ -123,10 +143,19 @@ struct DevDomain {
   long long nb;
   long long tiles_x, tiles_y, tiles_z, tiles_per_node;
   long long tile_begin;     // first global tile of this domain
+  FastDiv by_major;         // division by tiles_per_node (order 1) or nodes (order 0)
+  FastDiv by_txy, by_tx;    // division by tiles_x * tiles_y and by tiles_x
   long long bitem_begin;    // first global boundary item (node-major) of this domain
   long long runs_per_node;  // pitch / kRun
   long long run_begin;      // first global run of this domain
 };
+
+// The tile decode's divisions, from the tile counts of the domain.
+inline void set_tile_divisions(DevDomain& D, int order) {
+  D.by_major = fast_div((uint32_t)(order == 0 ? D.nodes : D.tiles_per_node));
+  D.by_txy = fast_div((uint32_t)(D.tiles_x * D.tiles_y));
+  D.by_tx = fast_div((uint32_t)D.tiles_x);
+}
 
 struct StepParams {
   int n_domains;
@@ -150,6 +179,9 @@ struct StepParams {
   int even_pair;               // 16-bit storage, BGK: even level two x-adjacent cells per thread,
                                // kernel sized for 2 or 3 resident blocks (0: one cell per thread)
   int bx, by, bz, order;
+  unsigned listed_blocks;      // blocks of a launch that carry the listed items, and the spacing
+  unsigned listed_every;       // of these blocks over the grid, with the division by it
+  FastDiv by_listed_every;
   // persistent mode
   unsigned int* bar_count;
   unsigned int* bar_gen;
