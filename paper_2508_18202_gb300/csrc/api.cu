@@ -408,6 +408,36 @@ void apply_tiling(sc_lbm_t h) {
   h->persist_grid = 0;
 }
 
+// The launch shape of a handle that is neither tuned nor given one.  Rows of
+// 32 cells waste the least on a width that is no multiple of the block, and
+// blocks of two rows leave the level's last wave short.  Even + odd level in us
+// against 64 x 2 x 8, BGK: 13 samples of 256 x 128 x 64 FP32 1357 -> 1310 at
+// 32 x 2 x 4, 3 of 512 x 256 x 128 2543 -> 2466, 13 of 97 x 61 x 33 164 -> 154
+// (32 x 2 x 2: 151), FP16 131 -> 127.  A thread walks its slab serially, so a
+// level that leaves the chip idle takes shorter ones: 13 of 64 x 40 x 24 59 -> 51
+// at 32 x 2 x 2 (4: 55), 3 of 45 x 21 x 14 28.7 -> 16.4 at 32 x 1 x 1 (32 x 2 x 2: 16.9).
+// The regularized collision carries more arithmetic per cell and gains from
+// longer slabs: 25 of 120 x 120 x 40 787 -> 762 at 32 x 4 x 8 (32 x 2 x 4: 771).
+sc_lbm_tuning default_tuning(const sc_lbm_t h) {
+  sc_lbm_tuning t;
+  t.variant = 0;
+  t.tile_order = 1;
+  t.exec_mode = SC_EXEC_LAUNCH;
+  t.graph_steps = 50;
+  if (h->cfg.precision == SC_P_FP64_PLAIN) {
+    t.block_x = 64, t.block_y = 2, t.slab_z = 8;
+    return t;
+  }
+  long long cells = 0;
+  for (int d = 0; d < h->P.n_domains; ++d) cells += h->P.dom[d].ncell * h->P.dom[d].nodes;
+  t.block_x = 32, t.block_y = 2;
+  if (cells < 200000) t.block_y = 1, t.slab_z = 1;
+  else if (cells < 4000000) t.slab_z = 2;
+  else if (h->cfg.collision == SC_COLL_RR) t.block_y = 4, t.slab_z = 8;
+  else t.slab_z = 4;
+  return t;
+}
+
 int check_tuning(const sc_lbm_tuning& t) {
   // the step kernels are compiled for at most 256 threads per block
   if (t.block_x < 32 || t.block_x % 32 || t.block_y < 1 || t.block_x * t.block_y > 256) return SC_ERR_ARG;
@@ -831,14 +861,7 @@ int sc_lbm_init(const sc_lbm_config* cfg, void* d_ws, size_t bytes, void* cuda_s
   h->tma_ok = c.precision != SC_P_FP64_PLAIN;
   for (int d = 0; d < c.n_domains; ++d)
     if (c.domains[d].nx % (int)(16 / storage_bytes(c.precision)) != 0) h->tma_ok = 0;
-  // default launch shape
-  h->tune.variant = 0;
-  h->tune.block_x = 64;
-  h->tune.block_y = 2;
-  h->tune.slab_z = 8;
-  h->tune.tile_order = 1;
-  h->tune.exec_mode = SC_EXEC_LAUNCH;
-  h->tune.graph_steps = 50;
+  h->tune = default_tuning(h);
   apply_tiling(h);
 
   auto up = [&](size_t off, const void* src, size_t n) {
