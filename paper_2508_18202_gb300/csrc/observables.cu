@@ -551,54 +551,120 @@ __global__ void average_add_kernel(const __grid_constant__ StepParams P, int dom
 // parts of grad u, by central differences (dx = 1) where both neighbours
 // along an axis are fluid, one-sided where one is, zero where none is;
 // periodic axes wrap; solid cells get 0.
-__device__ void qcriterion_cell(const DevDomain& D, const float* __restrict__ u, float* __restrict__ q,
-                                long long c) {
+//
+// sum_ia (W_ia^2 - S_ia^2) = -sum_ia J_ia J_ai, so Q is six products of the
+// velocity gradient J.  A difference of two floats is a float pair exactly
+// (TwoSum), and the products are summed as float pairs (the Dot2 scheme of
+// DF2 above), which carries Q to about 2^-45 of its terms before the one
+// rounding to float; GB300's FP64 pipe runs at 1/64 of the FP32 rate and the
+// same sums in FP64 kept it 85% busy.  J is scaled by a power of two to its
+// largest entry, so the pairs neither overflow nor lose their low parts.  Q
+// of one 256 x 128 x 64 field: 368 -> 42 us.
+struct Diff {
+  float hi, lo;
+};
+__device__ __forceinline__ Diff two_diff(float a, float b) {
+  Diff d;
+  d.hi = __fadd_rn(a, -b);
+  const float bb = __fadd_rn(d.hi, -a);
+  d.lo = __fadd_rn(__fadd_rn(a, -__fadd_rn(d.hi, -bb)), -__fadd_rn(b, bb));
+  return d;
+}
+
+// Q of a cell whose gradient has entries near the end of the float range or
+// beyond it, in FP64: J = (up - dn) f, f the axis' factor.
+__device__ __noinline__ float qcriterion_wide(const float up[3][3], const float dn[3][3], const float f[3]) {
+  double s2 = 0.0, w2 = 0.0;
+  for (int i = 0; i < 3; ++i)
+    for (int a = 0; a < 3; ++a) {
+      const double ja = (double)f[a] * ((double)up[i][a] - (double)dn[i][a]);
+      const double ji = (double)f[i] * ((double)up[a][i] - (double)dn[a][i]);
+      const double sv = 0.5 * (ja + ji), wv = 0.5 * (ja - ji);
+      s2 += sv * sv;
+      w2 += wv * wv;
+    }
+  return (float)(0.5 * (w2 - s2));
+}
+
+__global__ void __launch_bounds__(256) qcriterion_kernel(const __grid_constant__ StepParams P, int domain,
+                                                         const float* __restrict__ u, float* __restrict__ q) {
+  const DevDomain& D = P.dom[domain];
+  const int ncell = (int)D.ncell;  // 19 ncell < 2^31
+  const int c = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (c >= ncell) return;
   if (D.flags[c]) {
     q[c] = 0.0f;
     return;
   }
-  const int xyz[3] = {(int)(c % D.nx), (int)((c / D.nx) % D.ny), (int)(c / ((long long)D.nx * D.ny))};
-  const int dim[3] = {D.nx, D.ny, D.nz};
-  double J[3][3];  // J[i][a] = d u_i / d x_a
+  const int row = c / D.nx, x = c - row * D.nx, z = row / D.ny, y = row - z * D.ny;
+  const int pos[3] = {x, y, z}, dim[3] = {D.nx, D.ny, D.nz}, step[3] = {1, D.nx, D.nx * D.ny};
+  float up[3][3], dn[3][3], f[3];  // [component][axis]: the two ends of a difference, and its factor
+#pragma unroll
   for (int a = 0; a < 3; ++a) {
-    long long nb[2];
-    bool ok[2];
-    for (int sgn = 0; sgn < 2; ++sgn) {
-      int p[3] = {xyz[0], xyz[1], xyz[2]};
-      p[a] += sgn ? 1 : -1;
-      ok[sgn] = true;
-      if (p[a] < 0 || p[a] >= dim[a]) {
-        if (D.bc[2 * a] == SC_BC_PERIODIC) p[a] = (p[a] + dim[a]) % dim[a];
-        else ok[sgn] = false;
-      }
-      nb[sgn] = ok[sgn] ? cidx(D, p[0], p[1], p[2]) : c;
-      if (ok[sgn] && D.flags[nb[sgn]]) ok[sgn] = false;
-    }
+    const bool wrap = D.bc[2 * a] == SC_BC_PERIODIC;
+    const bool first = pos[a] == 0, last = pos[a] == dim[a] - 1;
+    const int lo = first ? c + (dim[a] - 1) * step[a] : c - step[a];
+    const int hi = last ? c - (dim[a] - 1) * step[a] : c + step[a];
+    const bool ok0 = (!first || wrap) && !D.flags[lo], ok1 = (!last || wrap) && !D.flags[hi];
+    const int c0 = ok0 ? lo : c, c1 = ok1 ? hi : c;
+    f[a] = ok0 && ok1 ? 0.5f : 1.0f;
+#pragma unroll
     for (int i = 0; i < 3; ++i) {
-      const float* ui = u + (long long)i * D.ncell;
-      double d = 0.0;
-      if (ok[0] && ok[1]) d = 0.5 * ((double)ui[nb[1]] - (double)ui[nb[0]]);
-      else if (ok[1]) d = (double)ui[nb[1]] - (double)ui[c];
-      else if (ok[0]) d = (double)ui[c] - (double)ui[nb[0]];
-      J[i][a] = d;
+      up[i][a] = u[i * ncell + c1];
+      dn[i][a] = u[i * ncell + c0];
     }
   }
-  double s2 = 0.0, w2 = 0.0;
+  Diff J[3][3];
+  float m = 0.0f;
+#pragma unroll
   for (int i = 0; i < 3; ++i)
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-      const double sv = 0.5 * (J[i][a] + J[a][i]), wv = 0.5 * (J[i][a] - J[a][i]);
-      s2 += sv * sv;
-      w2 += wv * wv;
+      J[i][a] = two_diff(up[i][a], dn[i][a]);
+      m = fmaxf(m, fabsf(J[i][a].hi));
     }
-  q[c] = (float)(0.5 * (w2 - s2));
-}
-
-__global__ void qcriterion_kernel(const __grid_constant__ StepParams P, int domain, const float* __restrict__ u,
-                                  float* __restrict__ q) {
-  const DevDomain& D = P.dom[domain];
-  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < D.ncell;
-       c += (long long)gridDim.x * blockDim.x)
-    qcriterion_cell(D, u, q, c);
+  bool wide = false;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) wide |= !(fabsf(J[i][a].hi) < 1e38f);  // NaN, infinite or about to overflow
+  if (wide) {
+    q[c] = qcriterion_wide(up, dn, f);
+    return;
+  }
+  if (m < 1e-37f) {  // zero or next to the subnormal numbers: Q is zero in a float
+    q[c] = 0.0f;
+    return;
+  }
+  // 2^-e with e the exponent of m: J 2^-e lies in (-2, 2)
+  const float sc = __int_as_float((254 << 23) - (__float_as_int(m) & 0x7f800000));
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      J[i][a].hi *= f[a] * sc;
+      J[i][a].lo *= f[a] * sc;
+    }
+  float hi = 0.0f, lo = 0.0f;
+  auto add = [&](const Diff& a, const Diff& b, float w) {  // += w a b, w = 1 or 2
+    const float ah = w * a.hi;
+    const float p = __fmul_rn(ah, b.hi);
+    const float e = __fmaf_rn(ah, b.hi, -p);
+    const float t = __fmaf_rn(ah, b.lo, __fmul_rn(w * a.lo, b.hi));
+    const float s = __fadd_rn(hi, p);
+    const float bb = __fadd_rn(s, -hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fadd_rn(hi, -__fadd_rn(s, -bb)), __fadd_rn(p, -bb)), __fadd_rn(e, t)));
+    hi = s;
+  };
+  add(J[0][0], J[0][0], 1.0f);
+  add(J[1][1], J[1][1], 1.0f);
+  add(J[2][2], J[2][2], 1.0f);
+  add(J[0][1], J[1][0], 2.0f);
+  add(J[0][2], J[2][0], 2.0f);
+  add(J[1][2], J[2][1], 2.0f);
+  // Q = -(hi + lo) / 2 times 2^2e, the scale in two factors (2^2e itself may overflow)
+  const float back = __int_as_float(__float_as_int(m) & 0x7f800000);
+  q[c] = (-0.5f * __fadd_rn(hi, lo)) * back * back;
 }
 
 // The quadrature moments from (possibly all-reduced) sums, as the moment
@@ -764,7 +830,7 @@ int launch_scale(const double* in, double s, double* out, long long n, void* str
 
 int launch_qcriterion(const StepParams& P, int domain, const float* u, float* q, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
-  qcriterion_kernel<<<grid_for(P.dom[domain].ncell, 256), 256, 0, s>>>(P, domain, u, q);
+  qcriterion_kernel<<<(unsigned)((P.dom[domain].ncell + 255) / 256), 256, 0, s>>>(P, domain, u, q);
   return (int)cudaGetLastError();
 }
 
