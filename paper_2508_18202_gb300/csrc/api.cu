@@ -47,7 +47,7 @@ struct DomLayout {
 struct Layout {
   size_t hdr = 0, probes = 0;
   size_t st_mean = 0, st_std = 0, st_coef = 0, st_prof = 0, st_pnodes = 0;
-  size_t q_phi = 0, q_cells = 0, q_k = 0;  // gPC quantile scratch (gpc_degree >= 0)
+  size_t q_phi = 0, q_phif = 0, q_cells = 0, q_k = 0;  // gPC quantile scratch (gpc_degree >= 0)
   DomLayout dom[kMaxDomains];
   size_t total = 0;
 };
@@ -211,6 +211,7 @@ int plan(const sc_lbm_config* c, Layout& L, std::string& why) {
   L.st_pnodes = take(sizeof(float) * (size_t)kMaxProbes * max_nq * max_nz);
   if (P > 0) {
     L.q_phi = take(sizeof(double) * (size_t)SC_QUANTILE_MAX_SAMPLES * P);
+    L.q_phif = take(sizeof(float) * (size_t)SC_QUANTILE_MAX_SAMPLES * P);
     L.q_cells = take(sizeof(int32_t) * (size_t)SC_QUANTILE_MAX_CELLS);
     L.q_k = take(sizeof(int32_t) * (size_t)SC_QUANTILE_MAX_Q);
   }
@@ -1080,6 +1081,9 @@ int sc_lbm_gpc_quantiles(sc_lbm_t h, int domain, const double* d_coef, int n_cel
                  h->cfg.quad_rule == SC_Q_GH);
   }
   if (n_cells == 0) return SC_OK;
+  double phi_max[kMaxGpcP] = {};
+  for (int m = 0; m < n_samples; ++m)
+    for (int a = 0; a < P; ++a) phi_max[a] = std::max(phi_max[a], std::fabs(phi[(size_t)m * P + a]));
   std::vector<int32_t> cl(cells, cells + n_cells);
   const Layout& L = h->L;
   // pageable sources: each copy has taken its data when the call returns
@@ -1087,7 +1091,7 @@ int sc_lbm_gpc_quantiles(sc_lbm_t h, int domain, const double* d_coef, int n_cel
   CK(cudaMemcpyAsync(h->ws + L.q_cells, cl.data(), sizeof(int32_t) * cl.size(), cudaMemcpyHostToDevice, h->stream));
   CK(cudaMemcpyAsync(h->ws + L.q_k, kidx.data(), sizeof(int32_t) * kidx.size(), cudaMemcpyHostToDevice, h->stream));
   const int rc = launch_gpc_quantiles(d_coef, D.ncell, P, (const int32_t*)(h->ws + L.q_cells), n_cells,
-                                      (const double*)(h->ws + L.q_phi), n_samples,
+                                      (const double*)(h->ws + L.q_phi), phi_max, (float*)(h->ws + L.q_phif), n_samples,
                                       (const int32_t*)(h->ws + L.q_k), n_q, d_out, h->stream);
   if (rc) return cuda_fail(h, (cudaError_t)rc, "quantile launch");
   ++h->launches;

@@ -274,8 +274,11 @@ int launch_scale(const double* in, double s, double* out, long long n, void* str
 int launch_qcriterion(const StepParams& P, int domain, const float* u, float* q, void* stream);
 // Confidence bounds from the gPC surrogate (quantiles.cu): per listed cell
 // the k-th smallest of sum_a coef[a][cell] phi[m][a] over the M samples.
+// phi_max: host [P], the largest |phi[m][a]| of each term; phif: device
+// scratch of P * (M rounded up to a multiple of 4) floats.
 int launch_gpc_quantiles(const double* coef, long long ncell, int P, const int32_t* cells, int n_cells,
-                         const double* phi, int M, const int32_t* kidx, int nq, double* out, void* stream);
+                         const double* phi, const double* phi_max, float* phif, int M, const int32_t* kidx, int nq,
+                         double* out, void* stream);
 int launch_check(const StepParams& P, int precision, unsigned long long* d_count, void* stream);
 
 // Adjoint of one node's time step (adjoint.cu).
