@@ -79,7 +79,7 @@ extern "C" {
 #define SC_PROFILE_LOG 1     /* u_ref (1 + xi) ln((h+z0)/z0) / ln((H+z0)/z0)   */
 
 /* population precision                                                       */
-#define SC_P_FP64_PLAIN 0    /* FP64, unshifted, two arrays, one node per launch */
+#define SC_P_FP64_PLAIN 0    /* FP64, unshifted, two arrays                     */
 #define SC_P_FP32_SHIFT 1    /* FP32 storing g_i = f_i - w_i, in place (AA)     */
 #define SC_P_BF16_STORE 2    /* BF16 storage of g_i, FP32 arithmetic            */
 #define SC_P_FP16_STORE 3    /* FP16 storage of g_i, FP32 arithmetic            */

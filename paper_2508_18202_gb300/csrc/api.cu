@@ -592,20 +592,15 @@ int run_persistent(sc_lbm_t h, long long t, int n, const Wind<double>& w) {
 }
 
 int run_plain(sc_lbm_t h, int n) {
-  for (int d = 0; d < h->P.n_domains; ++d)
-    for (int j = 0; j < h->P.dom[d].nodes; ++j) {
-      StepParams P = h->P;
-      P.plain_domain = d;
-      P.plain_node = j;
-      for (int s = 0; s < n; ++s) {
-        set_winds(h, P, h->steps + s);
-        int rc = h->cfg.collision == SC_COLL_RR
-                     ? rr::launch_plain_step(P, (unsigned long long)(h->steps + s), h->stream)
-                     : launch_plain_step(P, (unsigned long long)(h->steps + s), h->stream);
-        if (rc) return cuda_fail(h, (cudaError_t)rc, "plain_step launch");
-        ++h->launches;
-      }
-    }
+  StepParams P = h->P;
+  for (int s = 0; s < n; ++s) {
+    const unsigned long long lvl = (unsigned long long)(h->steps + s);
+    set_winds(h, P, (long long)lvl);
+    int rc = h->cfg.collision == SC_COLL_RR ? rr::launch_plain_step(P, lvl, h->stream)
+                                            : launch_plain_step(P, lvl, h->stream);
+    if (rc) return cuda_fail(h, (cudaError_t)rc, "plain_step launch");
+    ++h->launches;
+  }
   return SC_OK;
 }
 
@@ -765,6 +760,8 @@ int sc_lbm_init(const sc_lbm_config* cfg, void* d_ws, size_t bytes, void* cuda_s
   P.smag18c2 = (float)(18.0 * c.c_smag * c.c_smag);
   P.smag18c2_d = 18.0 * c.c_smag * c.c_smag;
   P.csmag_on = c.c_smag > 0 ? 1 : 0;
+  P.omega0 = 1.0f / P.tau0;
+  P.omega0_d = 1.0 / P.tau0_d;
   Header* H = h->hdr();
   P.err = &H->err;
   P.bar_count = &H->bar_count;

@@ -232,14 +232,14 @@ __device__ __forceinline__ double fma1(double a, double b, double c) { return __
 // populations are g = f - w.  The non-equilibrium stress uses the exact
 // second moment of the D3Q19 second-order equilibrium, rho/3 I + rho u u.
 template <class T, bool SHIFT>
-__device__ __forceinline__ void collide(T g[kQ], T tau0, T smag18c2, bool smag_on) {
+__device__ __forceinline__ void collide(T g[kQ], T tau0, T omega0, T smag18c2, bool smag_on) {
   T m0, jx, jy, jz, pxx, pyy, pzz, pxy, pxz, pyz;
   all_sums<T>(g, m0, jx, jy, jz, pxx, pyy, pzz, pxy, pxz, pyz);
   const T rho = SHIFT ? add1(T(1), m0) : m0;
   const T inv = recip(rho);
   const T ux = mul1(jx, inv), uy = mul1(jy, inv), uz = mul1(jz, inv);
   const T usq = fma1(uz, uz, fma1(ux, ux, mul1(uy, uy)));
-  T tau = tau0;
+  T omega = omega0;
   if (smag_on) {
     // Pi^neq = sum c c g - (m0/3 I + rho u u); m0 = rho - 1 (shifted) or rho
     const T rx = mul1(rho, ux), ry = mul1(rho, uy), rz = mul1(rho, uz);
@@ -252,9 +252,8 @@ __device__ __forceinline__ void collide(T g[kQ], T tau0, T smag18c2, bool smag_o
     const T dia = fma1(nzz, nzz, fma1(nxx, nxx, mul1(nyy, nyy)));
     const T off = fma1(nyz, nyz, fma1(nxy, nxy, mul1(nxz, nxz)));
     const T pin = sqrt(fma1(T(2), fma1(T(2), off, dia), T(1e-30)));
-    tau = mul1(T(0.5), add1(tau0, sqrt(fma1(tau0, tau0, mul1(mul1(smag18c2, pin), inv)))));
+    omega = recip(mul1(T(0.5), add1(tau0, sqrt(fma1(tau0, tau0, mul1(mul1(smag18c2, pin), inv))))));
   }
-  const T omega = recip(tau);
   // Opposite pairs (i, i + 1), i odd, share c_i . u up to the sign: the
   // bracket of the equilibrium splits into an even part
   // m0 + rho (4.5 cu^2 - 1.5 u^2) (m0: w (rho - 1) shifted, w rho plain) and
@@ -488,9 +487,9 @@ __device__ __forceinline__ void collide_p(const StepParams& P, T g[kQ]) {
     collide_rr<T, SHIFT>(g, T(P.tau0), T(P.smag18c2), P.csmag_on);
 #else
   if constexpr (sizeof(T) == 8)
-    collide<T, SHIFT>(g, T(P.tau0_d), T(P.smag18c2_d), P.csmag_on);
+    collide<T, SHIFT>(g, T(P.tau0_d), T(P.omega0_d), T(P.smag18c2_d), P.csmag_on);
   else
-    collide<T, SHIFT>(g, T(P.tau0), T(P.smag18c2), P.csmag_on);
+    collide<T, SHIFT>(g, T(P.tau0), T(P.omega0), T(P.smag18c2), P.csmag_on);
 #endif
 }
 

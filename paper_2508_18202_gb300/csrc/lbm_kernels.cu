@@ -882,66 +882,73 @@ __global__ void __launch_bounds__(256, 3) aa_persistent_kernel(const __grid_cons
 }
 
 // ------------------------------------------------------------ FP64 plain path
-// Two arrays, push form, one node per launch.  Blocks [0, tiles_per_node)
-// take the bulk cells, the rest the listed boundary cells.
-__global__ void __launch_bounds__(256) plain_step_kernel(const __grid_constant__ StepParams P,
-                                                         unsigned long long n) {
-  const DevDomain& D = P.dom[P.plain_domain];
-  const int node = P.plain_node;
-  const long long pc = D.pitch;
-  double* A = reinterpret_cast<double*>(D.g) + (long long)node * kQ * pc;
-  double* B = reinterpret_cast<double*>(D.g2) + (long long)node * kQ * pc;
-  const double* src = (n & 1ull) ? B : A;
-  double* dst = (n & 1ull) ? A : B;
-  const long long sy = D.nx, sz = (long long)D.nx * D.ny;
-  const long long b = blockIdx.x;
-  if (b < D.tiles_per_node) {
-    const int tx = (int)(b % D.tiles_x);
-    const int ty = (int)((b / D.tiles_x) % D.tiles_y);
-    const int tz = (int)(b / (D.tiles_x * D.tiles_y));
-    const int x = tx * P.bx + threadIdx.x;
-    const int y = ty * P.by + threadIdx.y;
-    if (x >= D.nx || y >= D.ny) return;
-    const int z0 = tz * P.bz, z1 = min(z0 + P.bz, D.nz);
-    Node<double> N;
-    N.g = dst;
-    N.bout = nullptr;
-    N.uinf = nullptr;
-    N.uind = D.uin_d + (long long)node * D.nz * 3;
-    for (int z = z0; z < z1; ++z) {
-      const long long idx = cidx(D, x, y, z);
-      const LinkWord lw = __ldg(D.link + idx);
-      if (lw & kLinkSlow) continue;
-      double g[kQ];
-#pragma unroll
-      for (int i = 0; i < kQ; ++i) g[i] = src[(long long)i * pc + idx];
-      collide_p<double, false>(P, g);
-      double ux, uy, uz;
-      wall_velocity<double>(N, lw, z, P.wqd, ux, uy, uz);
-      fast_push<double>(dst + idx, lw, (int)pc, (int)sy, (int)sz, ux, uy, uz, P.wqd.scale, g);
-    }
-    return;
-  }
-  const long long item = (b - D.tiles_per_node) * (long long)(P.bx * P.by) + threadIdx.y * P.bx + threadIdx.x;
-  if (item >= D.nb) return;
-  const long long idx = __ldg(D.bcell + item);
-  const int z = (int)(idx / ((long long)D.nx * D.ny));
-  const ListedRef L = listed_ref(D, item);
+// Two arrays, push form, every node of every domain in one launch.  The FP64
+// pipe bounds it (two lanes per cycle and SM), so the work is spread for that
+// pipe alone: threads take consecutive cells (no lanes lost to a row's end:
+// a 48-cell row would leave a quarter of a 64-wide tile's lanes idle in every
+// FP64 instruction), blocks of 128 threads share the last wave evenly, and
+// only the warps that have a moving-wall or specular link carry its FP64
+// terms.  The trailing blocks take the listed cells.  5 nodes of 48 x 24 x 24,
+// a time step: 400 us as one launch a node of 64 x 2 x 8 tiles (41 blocks on
+// 152 SMs), 59.5 us (FP64 pipe 81% busy); 2 of 128 x 64 x 48: 581 -> 370 us.
+constexpr int kPlainThreads = 128;
+
+__device__ __forceinline__ Node<double> plain_node(const DevDomain& D, double* dst, int node) {
   Node<double> N;
   N.g = dst;
   N.bout = nullptr;
   N.uinf = nullptr;
   N.uind = D.uin_d + (long long)node * D.nz * 3;
-  double g[kQ];
-#pragma unroll
-  for (int i = 0; i < kQ; ++i) g[i] = src[(long long)i * pc + idx];
-  collide_p<double, false>(P, g);
-  double ux = 0.0, uy = 0.0, uz = 0.0;
-  if (L.word(kWordPushMove)) inflow_velocity<double>(N, z, P.wqd, ux, uy, uz);
-  listed_push<double>(L, dst, ux, uy, uz, P.wqd.scale, g);
+  return N;
 }
 
-
+__global__ void __launch_bounds__(kPlainThreads) plain_step_kernel(const __grid_constant__ StepParams P,
+                                                                   unsigned long long n) {
+  constexpr unsigned kPer = kRun / kPlainThreads;  // blocks of a run
+  if (blockIdx.x < kPer * (unsigned)P.total_runs) {
+    const RunRef R = decode_run(P, blockIdx.x / kPer);
+    const DevDomain& D = P.dom[R.d];
+    const int pc = (int)D.pitch, sy = D.nx, sz = D.nx * D.ny;
+    const int c = (int)R.c0 + (int)(blockIdx.x % kPer) * kPlainThreads + (int)threadIdx.x;
+    const LinkWord lw = c < (int)D.ncell ? __ldg(D.link + c) : kLinkSolid;
+    const bool skip = (lw & kLinkSlow) != 0;
+    const bool general = __any_sync(0xffffffffu, !skip && (lw & kLinkGeneral));
+    if (skip) return;
+    const long long first = (long long)R.node * kQ * D.pitch;
+    double* const A = reinterpret_cast<double*>(D.g) + first;
+    double* const B = reinterpret_cast<double*>(D.g2) + first;
+    const double* src = (n & 1ull) ? B : A;
+    double* dst = (n & 1ull) ? A : B;
+    double g[kQ];
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) g[i] = src[i * pc + c];
+    collide_p<double, false>(P, g);
+    if (general) {
+      double ux, uy, uz;
+      wall_velocity<double>(plain_node(D, dst, R.node), lw, c / sz, P.wqd, ux, uy, uz);
+      mask_push<double, true>(dst + c, lw, pc, sy, sz, ux, uy, uz, P.wqd.scale, g);
+    } else {
+      mask_push<double, false>(dst + c, lw, pc, sy, sz, 0.0, 0.0, 0.0, 0.0, g);
+    }
+    return;
+  }
+  const long long item = (blockIdx.x - kPer * (unsigned)P.total_runs) * (long long)kPlainThreads + threadIdx.x;
+  if (item >= P.total_bitems) return;
+  int node;
+  long long idx;
+  const DevDomain& D = P.dom[decode_bitem(P, item, &node, &idx)];
+  const long long first = (long long)node * kQ * D.pitch;
+  const double* src = reinterpret_cast<const double*>((n & 1ull) ? D.g2 : D.g) + first;
+  double* dst = reinterpret_cast<double*>((n & 1ull) ? D.g : D.g2) + first;
+  const ListedRef L = listed_ref(D, (item - D.bitem_begin) % D.nb);
+  double g[kQ];
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) g[i] = src[(long long)i * D.pitch + idx];
+  collide_p<double, false>(P, g);
+  double ux = 0.0, uy = 0.0, uz = 0.0;
+  if (L.word(kWordPushMove)) inflow_velocity<double>(plain_node(D, dst, node), L.word(kWordZ), P.wqd, ux, uy, uz);
+  listed_push<double>(L, dst, ux, uy, uz, P.wqd.scale, g);
+}
 
 template <class S>
 size_t even_tma_smem() { return (size_t)kStages * kQ * kRun * sizeof(S) + 2 * kStages * sizeof(uint64_t); }
@@ -1107,13 +1114,9 @@ int launch_aa_persistent(const StepParams& P, int precision, void* stream, int g
 }
 
 int launch_plain_step(const StepParams& P, unsigned long long n, void* stream) {
-  const DevDomain& D = P.dom[P.plain_domain];
-  dim3 block(P.bx, P.by);
-  cudaStream_t s = (cudaStream_t)stream;
-  const long long threads = (long long)P.bx * P.by;
-  const long long grid = D.tiles_per_node + (D.nb + threads - 1) / threads;
   // the time level of the plain path is tracked on the host
-  plain_step_kernel<<<(unsigned)grid, block, 0, s>>>(P, n);
+  const long long grid = P.total_runs * (kRun / kPlainThreads) + (P.total_bitems + kPlainThreads - 1) / kPlainThreads;
+  plain_step_kernel<<<(unsigned)grid, kPlainThreads, 0, (cudaStream_t)stream>>>(P, n);
   return (int)cudaGetLastError();
 }
 

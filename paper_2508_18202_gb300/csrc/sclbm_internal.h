@@ -163,6 +163,8 @@ struct StepParams {
   float tau0;
   float smag18c2;             // 18 C_S^2
   double tau0_d, smag18c2_d;
+  float omega0;               // 1 / tau0, correctly rounded: the relaxation rate without the Smagorinsky term
+  double omega0_d;
   int csmag_on;
   unsigned long long n_host;  // time level of the state (observables, persistent start)
   // Inflow factors of the launch: wp at arrival level n (odd-level pulls,
@@ -188,8 +190,6 @@ struct StepParams {
   long long spin_limit;
   int never_arrive;
   int n_steps;                // persistent: steps per launch
-  int plain_node;             // FP64 plain path: node advanced by this launch
-  int plain_domain;
 };
 
 // ------------------------------------------------------------ host numerics
