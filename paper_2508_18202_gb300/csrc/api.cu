@@ -1536,7 +1536,7 @@ int sc_lbm_inflow_next_change(int ramp_steps, int n_targets, const double* speed
 // ------------------------------------------------------------ adjoint
 namespace {
 struct AdjLayout {
-  size_t accum, probes, target, uprobe, uin, du, lmap, states, state_bytes, total;
+  size_t accum, probes, target, uprobe, uin, du, states, state_bytes, total;
   int K, L;
 };
 
@@ -1561,7 +1561,6 @@ int adj_plan(sc_lbm_t h, int domain, int n_steps, int n_snapshots, int n_probes,
   A.uprobe = take(3 * sizeof(double) * (size_t)n_probes);
   A.uin = take(16 * (size_t)D.nz);
   A.du = take(32 * (size_t)D.nz);
-  A.lmap = take(sizeof(int32_t) * (size_t)D.ncell);
   A.state_bytes = align_up(sizeof(float) * kQ * (size_t)D.pitch);
   A.states = off;
   A.K = K;
@@ -1638,7 +1637,6 @@ int sc_lbm_adjoint(sc_lbm_t h, int domain, int node, const int32_t* probes, int 
   A.u_probe = (double*)(ws + L.uprobe);
   A.n_probes = n_probes;
   A.accum = (double*)(ws + L.accum);
-  A.lmap = (const int32_t*)(ws + L.lmap);
   auto state = [&](int k) { return (float*)(ws + L.states + L.state_bytes * (size_t)k); };
   float* snap0 = state(0);           // K checkpoints
   float* seg0 = state(L.K);          // L segment states
@@ -1652,40 +1650,42 @@ int sc_lbm_adjoint(sc_lbm_t h, int domain, int node, const int32_t* probes, int 
   // The device work of one gradient: forward sweep with checkpoints every L
   // steps from the equilibrium start, loss and seed at level T, then per
   // segment (last first) the recompute of its states and the reverse steps.
+  // The forward sweep writes each state where it is next read: a checkpoint
+  // straight into its place, the last segment's states into the segment
+  // buffers (that segment is not recomputed), the others into two buffers in
+  // turn; a segment's first state is read from its checkpoint.
   const size_t sf = L.state_bytes / sizeof(float);
+  const int last = (L.K - 1) * L.L;  // first level of the last segment
   auto issue = [&]() -> int {
     int r;
-    if ((r = ck(launch_adj_listed_map(P, domain, (int32_t*)(ws + L.lmap), h->stream), "adjoint map"))) return r;
-    if ((r = ck(launch_fill_zero(fa, nstate, h->stream), "adjoint fill"))) return r;
-    if ((r = ck(launch_fill_zero(fb, nstate, h->stream), "adjoint fill"))) return r;
-    float* cur = fa;
-    float* nxt = fb;
+    auto snap = [&](int k) { return snap0 + (size_t)k * sf; };
+    auto seg = [&](int k) { return seg0 + (size_t)k * sf; };
+    auto forward = [&](const float* src, float* dst, int n) {
+      return ck(launch_adj_forward(P, A, src, dst, (float)hn_ramp(h->cfg.ramp_steps, n + 1), h->stream),
+                "adjoint forward");
+    };
+    if ((r = ck(launch_fill_zero(snap0, nstate, h->stream), "adjoint fill"))) return r;
+    const float* cur = snap0;
     for (int n = 0; n < n_steps; ++n) {
-      if (n % L.L == 0)
-        CK(cudaMemcpyAsync(snap0 + (size_t)(n / L.L) * sf, cur, sizeof(float) * nstate, cudaMemcpyDeviceToDevice,
-                           h->stream));
-      if ((r = ck(launch_adj_forward(P, A, cur, nxt, (float)hn_ramp(h->cfg.ramp_steps, n + 1), h->stream),
-                  "adjoint forward")))
-        return r;
-      std::swap(cur, nxt);
+      float* next = cur == fa ? fb : fa;
+      if (n + 1 < n_steps && (n + 1) % L.L == 0) next = snap((n + 1) / L.L);
+      else if (n + 1 < n_steps && n + 1 > last) next = seg(n + 1 - last);
+      if ((r = forward(cur, next, n))) return r;
+      cur = next;
     }
     if ((r = ck(launch_fill_zero(lamA, nstate, h->stream), "adjoint fill"))) return r;
-    if ((r = ck(launch_fill_zero(lamB, nstate, h->stream), "adjoint fill"))) return r;
     if ((r = ck(launch_adj_loss(P, A, cur, lamA, h->stream), "adjoint loss"))) return r;
     float* lnext = lamA;
     float* lcur = lamB;
     for (int sgm = L.K - 1; sgm >= 0; --sgm) {
       const int n0 = sgm * L.L, n1 = std::min(n0 + L.L, n_steps);
-      CK(cudaMemcpyAsync(seg0, snap0 + (size_t)sgm * sf, sizeof(float) * nstate, cudaMemcpyDeviceToDevice,
-                         h->stream));
-      for (int n = n0; n < n1 - 1; ++n)
-        if ((r = ck(launch_adj_forward(P, A, seg0 + (size_t)(n - n0) * sf, seg0 + (size_t)(n - n0 + 1) * sf,
-                                       (float)hn_ramp(h->cfg.ramp_steps, n + 1), h->stream),
-                    "adjoint recompute")))
-          return r;
+      auto state_of = [&](int n) { return n == n0 ? snap(sgm) : seg(n - n0); };
+      if (n0 != last)
+        for (int n = n0; n < n1 - 1; ++n)
+          if ((r = forward(state_of(n), state_of(n + 1), n))) return r;
       for (int n = n1 - 1; n >= n0; --n) {
-        if ((r = ck(launch_adj_step(P, A, seg0 + (size_t)(n - n0) * sf, lnext, lcur,
-                                    (float)hn_ramp(h->cfg.ramp_steps, n + 1), h->stream),
+        if ((r = ck(launch_adj_step(P, A, state_of(n), lnext, lcur, (float)hn_ramp(h->cfg.ramp_steps, n + 1),
+                                    h->stream),
                     "adjoint step")))
           return r;
         std::swap(lnext, lcur);
@@ -1723,7 +1723,8 @@ int sc_lbm_adjoint(sc_lbm_t h, int domain, int node, const int32_t* probes, int 
     rc = issue();
     if (rc) return rc;
   }
-  h->launches += 2LL * n_steps + (n_steps - L.K) + 5;
+  // forward and reverse steps, the recomputed ones, and two fills and the loss
+  h->launches += 2LL * n_steps + (last - (L.K - 1)) + 3;
   double acc[3];
   CK(cudaMemcpyAsync(acc, ws + L.accum, sizeof acc, cudaMemcpyDeviceToHost, h->stream));
   if (u_probe_out)

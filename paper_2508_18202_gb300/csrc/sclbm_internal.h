@@ -291,7 +291,6 @@ struct AdjArgs {
   double* u_probe;        // [n_probes][3]
   int n_probes;
   double* accum;          // [0] loss, [1] dJ/du_ref, [2] dJ/dalpha
-  const int32_t* lmap;    // [ncell]: listed cell -> index in the listed-cell array
 };
 int launch_adj_forward(const StepParams& P, const AdjArgs& A, const float* src, float* dst, float r1,
                        void* stream);  // r1: ramp r(n + 1) of the step's pushes
@@ -299,6 +298,5 @@ int launch_adj_loss(const StepParams& P, const AdjArgs& A, const float* f, float
 int launch_adj_step(const StepParams& P, const AdjArgs& A, const float* f, const float* lam_next, float* lam,
                     float r1, void* stream);
 int launch_fill_zero(float* p, long long n, void* stream);
-int launch_adj_listed_map(const StepParams& P, int domain, int32_t* lmap, void* stream);
 
 }  // namespace sclbm
