@@ -959,6 +959,7 @@ int sc_lbm_moments(sc_lbm_t h, int domain, double* mean, double* stdev, const in
   A.stride = h->gpcP + 1;
   A.P = gpc_coef ? h->gpcP : 0;
   A.wsum = h->wsum[domain];
+  A.rwsum = 1.0 / A.wsum;
   A.mean = out_host ? (mean ? (double*)(h->ws + L.st_mean) : nullptr) : mean;
   A.stdev = out_host ? (stdev ? (double*)(h->ws + L.st_std) : nullptr) : stdev;
   A.coef = out_host ? (gpc_coef ? (double*)(h->ws + L.st_coef) : nullptr) : gpc_coef;
@@ -1008,6 +1009,7 @@ int sc_lbm_moment_sums(sc_lbm_t h, int domain, double* d_s1, double* d_s2, doubl
   A.stride = h->gpcP + 1;
   A.P = d_gpc_sums ? h->gpcP : 0;
   A.wsum = h->wsum[domain];
+  A.rwsum = 1.0 / A.wsum;
   A.mean = d_s1;
   A.stdev = d_s2;
   A.coef = d_gpc_sums;

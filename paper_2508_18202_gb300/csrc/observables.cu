@@ -74,6 +74,16 @@ __device__ __forceinline__ void gather_pops(const StepParams& P, const DevDomain
   }
 }
 
+// a / b with r = 1 / b correctly rounded: the quotient's residual by FMA
+// corrects it to the correctly rounded a / b (Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", IBM J. Res.
+// Develop. 34, 1990), so three quotients by one density cost one reciprocal.
+// (Below 2^-102 the residual may be inexact and the last bit differ.)
+__device__ __forceinline__ float quotient(float a, float b, float r) {
+  const float q = __fmul_rn(a, r);
+  return __fmaf_rn(__fmaf_rn(-b, q, a), r, q);
+}
+
 // Density and velocity from the populations gather_pops gives (Sec. 2.2:
 // rho = sum_i f_i, rho u = sum_i c_i f_i).  SHIFT: g_i = f_i - w_i, so
 // rho = 1 + sum_i g_i and, as sum_i w_i c_i = 0, rho u = sum_i c_i g_i; both
@@ -83,6 +93,15 @@ __device__ __forceinline__ void macro(const T g[kQ], T& rho, T& ux, T& uy, T& uz
   T m0, jx, jy, jz;
   flow_sums<T>(g, m0, jx, jy, jz);
   rho = SHIFT ? T(1) + m0 : m0;
+  if constexpr (sizeof(T) == 4) {
+    if (rho > 1e-18f && rho < 1e18f) {
+      const float r = recip(rho);
+      ux = quotient(jx, rho, r);
+      uy = quotient(jy, rho, r);
+      uz = quotient(jz, rho, r);
+      return;
+    }
+  }
   ux = jx / rho;
   uy = jy / rho;
   uz = jz / rho;
@@ -102,12 +121,31 @@ __device__ __forceinline__ T speed(T ux, T uy, T uz) {
     return __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(ux, ux), __dmul_rn(uy, uy)), __dmul_rn(uz, uz)));
 }
 
+// A float as a double by its bits: conversions run on the FP64 pipe, which
+// takes 16 cycles of an SM for each instruction of a warp and bounds the moment
+// kernels of a few nodes.  (Subnormal, infinite and NaN values are converted.)
+__device__ __forceinline__ double widen(float v) {
+  const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
+  if (m - 0x00800000u >= 0x7f000000u && m != 0u) return (double)v;
+  const uint32_t hi = (b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u);
+  return __hiloint2double((int)hi, (int)(b << 29));
+}
+
+// a / w with r = 1 / w correctly rounded, itself correctly rounded (as
+// quotient() above): three FP64 instructions instead of a division's dozen.
+__device__ __forceinline__ double quotient(double a, double w, double r) {
+  const double q = __dmul_rn(a, r);
+  if (((uint32_t)__double2hiint(q) & 0x7ff00000u) == 0x7ff00000u) return q;  // infinite or NaN: no residual
+  return __fma_rn(__fma_rn(-w, q, a), r, q);
+}
+
 // mean = S1 / W, std = sqrt(max(S2 / W - mean^2, 0)) (Eq. quad_moments; the
 // clamp guards negative sparse-grid weights), each operation rounded once so
 // that every kernel finishing sums gives the same bits for the same sums.
-__device__ __forceinline__ void finish_moments(double s1, double s2, double wsum, double& mean, double& sd) {
-  mean = __ddiv_rn(s1, wsum);
-  double var = __dsub_rn(__ddiv_rn(s2, wsum), __dmul_rn(mean, mean));
+// rw = 1 / W, correctly rounded.
+__device__ __forceinline__ void finish_moments(double s1, double s2, double wsum, double rw, double& mean, double& sd) {
+  mean = quotient(s1, wsum, rw);
+  double var = __dsub_rn(quotient(s2, wsum, rw), __dmul_rn(mean, mean));
   if (var < 0.0) var = 0.0;
   sd = __dsqrt_rn(var);
 }
@@ -161,7 +199,15 @@ __device__ __forceinline__ DF df_from(double v) {
   s.lo = __double2float_rn(v - (double)s.hi);
   return s;
 }
-__device__ __forceinline__ double df_value(DF s) { return (double)s.hi + (double)s.lo; }
+__device__ __forceinline__ double df_value(DF s) { return widen(s.hi) + widen(s.lo); }
+
+// The pair sums of terms a, a + 1 of cell c from the stored sums.
+__device__ __forceinline__ void df2_load(DF2& s, const MomentArgs& A, int a, int ncell, int c) {
+  const DF u = df_from(a < A.P ? A.coef[(long long)a * ncell + c] : 0.0);
+  const DF v = df_from(a + 1 < A.P ? A.coef[(long long)(a + 1) * ncell + c] : 0.0);
+  s.hi = make_float2(u.hi, v.hi);
+  s.lo = make_float2(u.lo, v.lo);
+}
 
 // Ensemble statistics of |u| per cell (Eq. quad_moments) and the gPC
 // projection (Eq. coef_discrete): one thread per cell runs over the nodes in
@@ -218,7 +264,7 @@ __global__ void __launch_bounds__(256) moments_kernel(const __grid_constant__ St
       A.mean[c] = s1;
       A.stdev[c] = s2;
     } else {
-      finish_moments(s1, s2, A.wsum, A.mean[c], A.stdev[c]);
+      finish_moments(s1, s2, A.wsum, A.rwsum, A.mean[c], A.stdev[c]);
     }
     if (A.coef) {
 #pragma unroll
@@ -228,6 +274,64 @@ __global__ void __launch_bounds__(256) moments_kernel(const __grid_constant__ St
   }
   const unsigned any = __ballot_sync(0xffffffffu, bad);
   if (any && (threadIdx.x & 31) == 0) atomicOr(P.err, kErrDiverged);
+}
+
+// How a warp's cells supply their populations of the current level, the same
+// at every node: the natural layout of an even level; at an odd level all
+// links streaming, or some cell with a wall, inflow, lid or listed link.
+// Decided once a warp before the loop over the nodes, so that the loop of an
+// all-streaming warp carries plain neighbour loads (decoding the link kinds of
+// every node was two thirds of the odd level's instructions).  A third odd form
+// for warps whose links only stream or bounce back costs more registers than
+// it saves (odd level of the 13-sample LES block 0.96 -> 1.25 ms).
+enum class Pops { kEven, kStream, kLinks };
+
+// |u| from a cell's populations, and whether they are of a diverged state.
+__device__ __forceinline__ float pops_speed(const float g[kQ], bool& bad) {
+  float rho, ux, uy, uz;
+  macro<float, true>(g, rho, ux, uy, uz);
+  if (!(rho > 0.0f) || !isfinite(ux + uy + uz) || !isfinite(rho)) bad = true;
+  return speed<float>(ux, uy, uz);
+}
+
+// |u| of one cell at one node: g0 the node's population base; listed: the
+// cell's record where it is a listed one.
+template <class S, Pops FORM>
+__device__ __forceinline__ float cell_speed(const StepParams& P, const DevDomain& D, int node, const S* g0, int c,
+                                            LinkWord lw, long long listed, bool& bad) {
+  float g[kQ];
+  // hidden from the optimiser per node: hoisted out of the node loop the 19
+  // row offsets would hold (and spill) 19 registers
+  int pc = (int)D.pitch, sy = D.nx, sz = D.nx * D.ny;
+  asm volatile("" : "+r"(pc), "+r"(sy), "+r"(sz));
+  if constexpr (FORM == Pops::kLinks) {
+    // P.wp is the inflow factor of the level
+    const Node<S> N = node_view<S>(D, node);
+    const int z = c / sz;
+    float ux, uy, uz;
+    if (lw & kLinkSlow) {
+      inflow_velocity<S>(N, z, P.wp, ux, uy, uz);
+      listed_pull<S, false>(listed_ref(D, listed), N.g, N.bout, ux, uy, uz, P.wp.scale, g);
+    } else {
+      wall_velocity<S>(N, lw, z, P.wp, ux, uy, uz);
+      mask_pull<S, false, true>(g0 + c, lw, pc, sy, sz, ux, uy, uz, P.wp.scale, g);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < kQ; ++i)
+      g[i] = Store<S>::ld(g0 + c + (FORM == Pops::kEven ? i * pc : OPP(i) * pc - (CX(i) + CY(i) * sy + CZ(i) * sz)));
+  }
+  return pops_speed(g, bad);
+}
+
+// f(form) with the form of the warp: lw is the link word of the lane's cell,
+// kLinkSolid beyond the domain.  ODD: the level's parity, a template argument
+// of the kernels so that the even level's holds no registers for the links.
+template <bool ODD, class F>
+__device__ __forceinline__ void with_pops_form(LinkWord lw, F&& f) {
+  if constexpr (!ODD) f(std::integral_constant<Pops, Pops::kEven>{});
+  else if (__all_sync(0xffffffffu, lw == 0 || (lw & kLinkSolid))) f(std::integral_constant<Pops, Pops::kStream>{});
+  else f(std::integral_constant<Pops, Pops::kLinks>{});
 }
 
 // The same statistics for the in-place precisions (|u| of the current level
@@ -242,68 +346,68 @@ __global__ void __launch_bounds__(256) moments_kernel(const __grid_constant__ St
 // agrees with one reduction over all nodes to the pairs' 48-bit rounding.
 // This form serves the small bases (PM <= kMomCellMaxP); a large basis holds
 // too many accumulators per thread for it and goes to moments_split_kernel.
-// Up to 10 terms three blocks are resident per SM (80 registers): at 10 terms
-// left to itself the compiler takes 128 registers and two blocks, 6.51 against
-// 5.15 ms on 12 samples of 512 x 256 x 128.
+// Up to 10 terms three blocks are resident per SM (80 registers).
+// Bound: the FP64 pipe where the nodes are few (16 cycles of an SM for an
+// instruction of a warp), so conversions go by the bits, the sums are only
+// converted where they continue, and a mean divides by a reciprocal; else the
+// latency of a node's loads and chains.  Even / odd level, with gPC sums: 13
+// samples of 256 x 128 x 64 670 / 1239 -> 419 / 965 us (FP32; BF16 670 / 1361 ->
+// 391 / 899), 6 of 512 x 256 x 128 3.73 / 5.07 -> 2.44 / 3.41 ms.
 constexpr int kMomCellMaxP = 12;
 
-template <class S, int PM>
+template <class S, int PM, bool ODD>
 __global__ void __launch_bounds__(256, PM <= 10 ? 3 : 2) moments_pair_kernel(const __grid_constant__ StepParams P, MomentArgs A) {
-  using T = typename Store<S>::C;
   constexpr int NP = PM > 0 ? PM / 2 : 1;
   const DevDomain& D = P.dom[A.domain];
-  const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const int c = (int)(blockIdx.x * blockDim.x + threadIdx.x);  // 19 ncell < 2^31
+  const int ncell = (int)D.ncell;
+  const bool inside = c < ncell;
+  const LinkWord lw = inside ? __ldg(D.link + c) : kLinkSolid;
+  const bool fluid = !(lw & kLinkSolid);
+  const bool acc = inside && A.raw && A.accumulate;
+  double s1 = acc ? A.mean[c] : 0.0, s2 = acc ? A.stdev[c] : 0.0;
+  DF2 cf[NP];
+#pragma unroll
+  for (int k = 0; k < NP; ++k) cf[k].hi = cf[k].lo = make_float2(0.0f, 0.0f);
+  if (acc && A.P > 0) {
+#pragma unroll
+    for (int k = 0; k < NP; ++k) df2_load(cf[k], A, 2 * k, ncell, c);
+  }
   bool bad = false;
-  if (c < D.ncell) {
-    const unsigned long long n = P.n_host;
-    const int x = (int)(c % D.nx);
-    const int y = (int)((c / D.nx) % D.ny);
-    const int z = (int)(c / ((long long)D.nx * D.ny));
-    const LinkWord lw = __ldg(D.link + c);
-    const bool acc = A.raw && A.accumulate;
-    double s1 = acc ? A.mean[c] : 0.0, s2 = acc ? A.stdev[c] : 0.0;
-    DF2 cf[NP];
+  with_pops_form<ODD>(lw, [&](auto form) {
+    if (!fluid) return;
+    constexpr Pops FORM = decltype(form)::value;
+    const long long listed = FORM == Pops::kLinks && (lw & kLinkSlow) ? listed_index(D, c) : 0;
+    const float4* bf = A.abf;
+    const double* ab = A.ab;
+    const S* g0 = reinterpret_cast<const S*>(D.g);
+    const long long next = (long long)kQ * D.pitch;
+    for (int j = 0; j < A.nq; ++j, bf += NP, ab += A.stride, g0 += next) {
+      const float qf = cell_speed<S, FORM>(P, D, j, g0, c, lw, listed, bad);
+      const double q = widen(qf);
+      const double aq = __ldg(ab) * q;
+      s1 += aq;
+      s2 = fma(aq, q, s2);
+      if constexpr (PM > 0) {
+        const float2 q2 = make_float2(qf, qf);
 #pragma unroll
-    for (int k = 0; k < NP; ++k) {
-      const int a = 2 * k;
-      const DF u = df_from((acc && a < A.P) ? A.coef[(long long)a * D.ncell + c] : 0.0);
-      const DF v = df_from((acc && a + 1 < A.P) ? A.coef[(long long)(a + 1) * D.ncell + c] : 0.0);
-      cf[k].hi = make_float2(u.hi, v.hi);
-      cf[k].lo = make_float2(u.lo, v.lo);
-    }
-    if (!(lw & kLinkSolid)) {
-      const float4* bf = A.abf;
-      const double* ab = A.ab;
-      for (int j = 0; j < A.nq; ++j, bf += NP, ab += A.stride) {
-        T g[kQ];
-        gather_pops<S, true>(P, D, j, n, x, y, z, c, lw, g);
-        T rho, ux, uy, uz;
-        macro<T, true>(g, rho, ux, uy, uz);
-        if (!(rho > T(0)) || !isfinite(ux + uy + uz) || !isfinite(rho)) bad = true;
-        const float qf = speed<T>(ux, uy, uz);
-        const double q = double(qf);
-        const double aq = __ldg(ab) * q;
-        s1 += aq;
-        s2 = fma(aq, q, s2);
-        if constexpr (PM > 0) {
-          const float2 q2 = make_float2(qf, qf);
-#pragma unroll
-          for (int k = 0; k < NP; ++k) df2_dot_add(cf[k], __ldg(bf + k), q2);
-        }
+        for (int k = 0; k < NP; ++k) df2_dot_add(cf[k], __ldg(bf + k), q2);
       }
     }
+  });
+  if (inside) {
     if (A.raw) {
       A.mean[c] = s1;
       A.stdev[c] = s2;
     } else {
-      finish_moments(s1, s2, A.wsum, A.mean[c], A.stdev[c]);
+      finish_moments(s1, s2, A.wsum, A.rwsum, A.mean[c], A.stdev[c]);
     }
     if (A.coef) {
 #pragma unroll
       for (int k = 0; k < NP; ++k) {
         const int a = 2 * k;
-        if (a < A.P) A.coef[(long long)a * D.ncell + c] = df_value(DF{cf[k].hi.x, cf[k].lo.x});
-        if (a + 1 < A.P) A.coef[(long long)(a + 1) * D.ncell + c] = df_value(DF{cf[k].hi.y, cf[k].lo.y});
+        if (a < A.P) A.coef[(long long)a * ncell + c] = df_value(DF{cf[k].hi.x, cf[k].lo.x});
+        if (a + 1 < A.P) A.coef[(long long)(a + 1) * ncell + c] = df_value(DF{cf[k].hi.y, cf[k].lo.y});
       }
     }
   }
@@ -327,16 +431,16 @@ __global__ void __launch_bounds__(256, PM <= 10 ? 3 : 2) moments_pair_kernel(con
 // the accumulators.  PM = gpc_pair_pad(A.P) is the padded basis size (a
 // multiple of 4) and the row length of A.abf; its pad terms are zero and are
 // not written.  raw and accumulate as in moments_pair_kernel; the two forms
-// give the same bits (measured on 6-, 10- and 21-term bases).  Three blocks per SM (80 registers, a few bytes
+// give the same bits (measured on 6-, 10- and 21-term bases).  121 samples of
+// 96 x 96 x 40, 21 terms, even / odd level: 1.23 / 1.61 -> 0.98 / 1.27 ms.  Three blocks per SM (80 registers, a few bytes
 // spilled at the largest bases) beat two unspilled ones: the wait on
 // dependent loads and arithmetic, not the instruction count, bounds this
 // reduction.
 constexpr int kMomPairs = 4;  // warp pairs per block (256 threads, 128 cells)
 
-template <class S, int PM>
+template <class S, int PM, bool ODD>
 __global__ void __launch_bounds__(64 * kMomPairs, 3) moments_split_kernel(const __grid_constant__ StepParams P,
                                                                          MomentArgs A) {
-  using T = typename Store<S>::C;
   static_assert(PM % 4 == 0, "two packed pairs of terms per thread pair");
   constexpr int NH = PM > 0 ? PM / 4 : 1;  // packed pairs per thread
   // the values a warp hands to its partner: [buffer][pair][warp of the pair][lane]
@@ -347,73 +451,65 @@ __global__ void __launch_bounds__(64 * kMomPairs, 3) moments_split_kernel(const 
   const int lane = threadIdx.x & 31;
   const int k = (threadIdx.x >> 5) & 1;  // 0: node j, S1, terms [0, PM/2); 1: node j + 1, S2, the rest
   const int pr = threadIdx.x >> 6;
-  const long long c = (blockIdx.x * (long long)kMomPairs + pr) * 32 + lane;
-  const bool inside = c < D.ncell;
-  int x = 0, y = 0, z = 0;
-  LinkWord lw = kLinkSolid;
-  if (inside) {
-    x = (int)(c % D.nx);
-    y = (int)((c / D.nx) % D.ny);
-    z = (int)(c / ((long long)D.nx * D.ny));
-    lw = __ldg(D.link + c);
-  }
-  const bool fluid = inside && !(lw & kLinkSolid);
-  const unsigned long long n = P.n_host;
-  const bool acc = A.raw && A.accumulate;
-  double s = (inside && acc) ? (k == 0 ? A.mean[c] : A.stdev[c]) : 0.0;
+  const int c = (int)((blockIdx.x * kMomPairs + pr) * 32 + lane);
+  const int ncell = (int)D.ncell;
+  const bool inside = c < ncell;
+  const LinkWord lw = inside ? __ldg(D.link + c) : kLinkSolid;
+  const bool fluid = !(lw & kLinkSolid);
+  const bool acc = inside && A.raw && A.accumulate;
+  double s = acc ? (k == 0 ? A.mean[c] : A.stdev[c]) : 0.0;
   DF2 cf[NH];
 #pragma unroll
-  for (int t = 0; t < NH; ++t) {
-    const int a = 2 * (k * NH + t);
-    const DF u = df_from((inside && acc && a < A.P) ? A.coef[(long long)a * D.ncell + c] : 0.0);
-    const DF v = df_from((inside && acc && a + 1 < A.P) ? A.coef[(long long)(a + 1) * D.ncell + c] : 0.0);
-    cf[t].hi = make_float2(u.hi, v.hi);
-    cf[t].lo = make_float2(u.lo, v.lo);
+  for (int t = 0; t < NH; ++t) cf[t].hi = cf[t].lo = make_float2(0.0f, 0.0f);
+  if (acc && A.P > 0) {
+#pragma unroll
+    for (int t = 0; t < NH; ++t) df2_load(cf[t], A, 2 * (k * NH + t), ncell, c);
   }
   bool bad = false;
   int buf = 0;
-  for (int j = 0; j < A.nq; j += 2, buf ^= 1) {
-    const int jn = j + k;  // the node this warp evaluates
-    const bool two = j + 1 < A.nq;
-    float qf = 0.0f;
-    double q = 0.0, aq = 0.0;
-    if (fluid && jn < A.nq) {
-      T g[kQ];
-      gather_pops<S, true>(P, D, jn, n, x, y, z, c, lw, g);
-      T rho, ux, uy, uz;
-      macro<T, true>(g, rho, ux, uy, uz);
-      if (!(rho > T(0)) || !isfinite(ux + uy + uz) || !isfinite(rho)) bad = true;
-      qf = speed<T>(ux, uy, uz);
-      q = double(qf);
-      aq = __ldg(A.ab + (long long)jn * A.stride) * q;
-    }
-    x_qf[buf][pr][k][lane] = qf;
-    x_q[buf][pr][k][lane] = q;
-    x_aq[buf][pr][k][lane] = aq;
-    // the two warps of the pair meet (named barrier 1 + pr, 64 threads); the
-    // alternating buffers keep the next exchange from overwriting this one
-    asm volatile("bar.sync %0, 64;" ::"r"(1 + pr) : "memory");
-    const float qf_o = x_qf[buf][pr][k ^ 1][lane];
-    const double q_o = x_q[buf][pr][k ^ 1][lane];
-    const double aq_o = x_aq[buf][pr][k ^ 1][lane];
-    const float qf0 = k ? qf_o : qf, qf1 = k ? qf : qf_o;
-    const double aq0 = k ? aq_o : aq, aq1 = k ? aq : aq_o;
-    if (fluid) {
-      s = fma(aq0, k ? q_o : 1.0, s);
-      if (two) s = fma(aq1, k ? q : 1.0, s);
-      if constexpr (PM > 0) {
-        const float4* b = A.abf + (long long)j * (PM / 2) + k * NH;
-        const float2 q0 = make_float2(qf0, qf0);
+  with_pops_form<ODD>(lw, [&](auto form) {
+    constexpr Pops FORM = decltype(form)::value;
+    const long long listed = FORM == Pops::kLinks && fluid && (lw & kLinkSlow) ? listed_index(D, c) : 0;
+    const long long next = (long long)kQ * D.pitch;
+    const S* g0 = reinterpret_cast<const S*>(D.g) + k * next;
+    for (int j = 0; j < A.nq; j += 2, buf ^= 1, g0 += 2 * next) {
+      const int jn = j + k;  // the node this warp evaluates
+      const bool two = j + 1 < A.nq;
+      float qf = 0.0f;
+      double q = 0.0, aq = 0.0;
+      if (fluid && jn < A.nq) {
+        qf = cell_speed<S, FORM>(P, D, jn, g0, c, lw, listed, bad);
+        q = widen(qf);
+        aq = __ldg(A.ab + (long long)jn * A.stride) * q;
+      }
+      x_qf[buf][pr][k][lane] = qf;
+      x_q[buf][pr][k][lane] = q;
+      x_aq[buf][pr][k][lane] = aq;
+      // the two warps of the pair meet (named barrier 1 + pr, 64 threads); the
+      // alternating buffers keep the next exchange from overwriting this one
+      asm volatile("bar.sync %0, 64;" ::"r"(1 + pr) : "memory");
+      const float qf_o = x_qf[buf][pr][k ^ 1][lane];
+      const double q_o = x_q[buf][pr][k ^ 1][lane];
+      const double aq_o = x_aq[buf][pr][k ^ 1][lane];
+      const float qf0 = k ? qf_o : qf, qf1 = k ? qf : qf_o;
+      const double aq0 = k ? aq_o : aq, aq1 = k ? aq : aq_o;
+      if (fluid) {
+        s = fma(aq0, k ? q_o : 1.0, s);
+        if (two) s = fma(aq1, k ? q : 1.0, s);
+        if constexpr (PM > 0) {
+          const float4* b = A.abf + (long long)j * (PM / 2) + k * NH;
+          const float2 q0 = make_float2(qf0, qf0);
 #pragma unroll
-        for (int t = 0; t < NH; ++t) df2_dot_add(cf[t], __ldg(b + t), q0);
-        if (two) {
-          const float2 q1 = make_float2(qf1, qf1);
+          for (int t = 0; t < NH; ++t) df2_dot_add(cf[t], __ldg(b + t), q0);
+          if (two) {
+            const float2 q1 = make_float2(qf1, qf1);
 #pragma unroll
-          for (int t = 0; t < NH; ++t) df2_dot_add(cf[t], __ldg(b + PM / 2 + t), q1);
+            for (int t = 0; t < NH; ++t) df2_dot_add(cf[t], __ldg(b + PM / 2 + t), q1);
+          }
         }
       }
     }
-  }
+  });
   x_q[buf][pr][k][lane] = s;
   asm volatile("bar.sync %0, 64;" ::"r"(1 + pr) : "memory");
   const double s_o = x_q[buf][pr][k ^ 1][lane];
@@ -423,15 +519,15 @@ __global__ void __launch_bounds__(64 * kMomPairs, 3) moments_split_kernel(const 
         A.mean[c] = s;
         A.stdev[c] = s_o;
       } else {
-        finish_moments(s, s_o, A.wsum, A.mean[c], A.stdev[c]);
+        finish_moments(s, s_o, A.wsum, A.rwsum, A.mean[c], A.stdev[c]);
       }
     }
     if (A.coef) {
 #pragma unroll
       for (int t = 0; t < NH; ++t) {
         const int a = 2 * (k * NH + t);
-        if (a < A.P) A.coef[(long long)a * D.ncell + c] = df_value(DF{cf[t].hi.x, cf[t].lo.x});
-        if (a + 1 < A.P) A.coef[(long long)(a + 1) * D.ncell + c] = df_value(DF{cf[t].hi.y, cf[t].lo.y});
+        if (a < A.P) A.coef[(long long)a * ncell + c] = df_value(DF{cf[t].hi.x, cf[t].lo.x});
+        if (a + 1 < A.P) A.coef[(long long)(a + 1) * ncell + c] = df_value(DF{cf[t].hi.y, cf[t].lo.y});
       }
     }
   }
@@ -480,7 +576,7 @@ __global__ void profiles_kernel(const __grid_constant__ StepParams P, MomentArgs
   }
   if (lane == 0) {
     double mean, sd;
-    finish_moments(s1, s2, A.wsum, mean, sd);
+    finish_moments(s1, s2, A.wsum, A.rwsum, mean, sd);
     double* out = A.prof + ((long long)p * D.nz + z) * 4;
     out[0] = mean;
     out[1] = sd;
@@ -669,10 +765,10 @@ __global__ void __launch_bounds__(256) qcriterion_kernel(const __grid_constant__
 
 // The quadrature moments from (possibly all-reduced) sums, as the moment
 // kernel finishes them.
-__global__ void finalize_moments_kernel(const double* __restrict__ s1, const double* __restrict__ s2, double wsum,
+__global__ void finalize_moments_kernel(const double* __restrict__ s1, const double* __restrict__ s2, double wsum, double rw,
                                         double* __restrict__ mean, double* __restrict__ stdev, long long n) {
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x)
-    finish_moments(s1[c], s2[c], wsum, mean[c], stdev[c]);
+    finish_moments(s1[c], s2[c], wsum, rw, mean[c], stdev[c]);
 }
 
 __global__ void scale_kernel(const double* __restrict__ in, double sc, double* __restrict__ out, long long n) {
@@ -748,10 +844,12 @@ int launch_moments(const StepParams& P, int precision, const MomentArgs& A, void
       auto pair = [&](auto pm) {
         constexpr int PM = decltype(pm)::value;
         if constexpr (SH && PM <= kMomCellMaxP) {
-          moments_pair_kernel<S, PM><<<grid, blk, 0, s>>>(P, A);
+          if (P.n_host & 1ull) moments_pair_kernel<S, PM, true><<<grid, blk, 0, s>>>(P, A);
+          else moments_pair_kernel<S, PM, false><<<grid, blk, 0, s>>>(P, A);
         } else if constexpr (SH) {
           const unsigned g2 = (unsigned)((D.ncell + 32 * kMomPairs - 1) / (32 * kMomPairs));  // two threads a cell
-          moments_split_kernel<S, PM><<<g2, 64 * kMomPairs, 0, s>>>(P, A);
+          if (P.n_host & 1ull) moments_split_kernel<S, PM, true><<<g2, 64 * kMomPairs, 0, s>>>(P, A);
+          else moments_split_kernel<S, PM, false><<<g2, 64 * kMomPairs, 0, s>>>(P, A);
         }
       };
       auto go = [&](auto avg) {
@@ -819,7 +917,7 @@ int launch_average_add(const StepParams& P, int precision, int domain, double* a
 
 int launch_finalize_moments(const double* s1, const double* s2, double wsum, double* mean, double* stdev,
                             long long n, void* stream) {
-  finalize_moments_kernel<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(s1, s2, wsum, mean, stdev, n);
+  finalize_moments_kernel<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(s1, s2, wsum, 1.0 / wsum, mean, stdev, n);
   return (int)cudaGetLastError();
 }
 

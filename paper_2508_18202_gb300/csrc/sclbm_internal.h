@@ -247,7 +247,7 @@ struct MomentArgs {
                            // (hi_a, hi_a+1, lo_a, lo_a+1) floats, hi + lo to 48 bits; zero pad terms
   int stride;              // row length of ab (basis size of the configuration + 1)
   int nq, P;               // P: coefficients to produce (0 = none)
-  double wsum;
+  double wsum, rwsum;      // sum of the weights, and 1 / wsum correctly rounded
   double* mean;
   double* stdev;
   double* coef;            // [P][ncell] or null
