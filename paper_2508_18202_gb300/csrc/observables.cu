@@ -219,7 +219,9 @@ __device__ __forceinline__ void df2_load(DF2& s, const MomentArgs& A, int a, int
 // the sums start from the values in the output arrays, so node ranges reduced
 // one after another (waves, shards) continue one sum per cell and carry the
 // bits of one reduction over all nodes.
-// AVG: the per-node time averages (A.avg) instead of the current |u|.
+// AVG: the per-node time averages (A.avg) instead of the current |u|.  Bound:
+// the FP64 pipe (90% busy), so what it need not do it does not: 13 samples of
+// 192 x 96 x 64, 6 terms: 413 -> 305 us.
 template <class S, bool SHIFT, int PM, bool AVG>
 __global__ void __launch_bounds__(256) moments_kernel(const __grid_constant__ StepParams P, MomentArgs A) {
   using T = typename Store<S>::C;
@@ -241,8 +243,8 @@ __global__ void __launch_bounds__(256) moments_kernel(const __grid_constant__ St
       for (int j = 0; j < A.nq; ++j) {
         double q;
         if constexpr (AVG) {
-          q = A.avg[(long long)j * D.ncell + c] * A.avg_scale;
-          if (!isfinite(q)) bad = true;
+          q = A.avg[(long long)j * D.ncell + c];
+          if (((uint32_t)__double2hiint(q) & 0x7ff00000u) == 0x7ff00000u) bad = true;  // infinite or NaN
         } else {
           T g[kQ];
           gather_pops<S, SHIFT>(P, D, j, n, x, y, z, c, lw, g);
@@ -259,6 +261,12 @@ __global__ void __launch_bounds__(256) moments_kernel(const __grid_constant__ St
         for (int a = 0; a < PM; ++a)
           if (a < A.P) coef[a] = fma(ab[1 + a], q, coef[a]);
       }
+    }
+    if constexpr (AVG) {  // the sums ran over the accumulators: one scale a sum instead of one a node
+      s1 *= A.avg_scale;
+      s2 *= A.avg_scale * A.avg_scale;
+#pragma unroll
+      for (int a = 0; a < PM; ++a) coef[a] *= A.avg_scale;
     }
     if (A.raw) {
       A.mean[c] = s1;
@@ -617,28 +625,33 @@ __global__ void export_kernel(const __grid_constant__ StepParams P, int domain, 
   }
 }
 
-// Count cells whose stored populations sum to a non-finite or non-positive
-// density (layout-independent: the stored 19 values of a cell always carry
-// its density at the current or previous time level).
 // Time average of |u| (the paper's time-averaged velocity magnitude fields,
 // Sec. 2.4 step 6): adds |u| at the current level, per (node, cell), in FP64.
-template <class S, bool SHIFT>
-__global__ void average_add_kernel(const __grid_constant__ StepParams P, int domain, double* avg) {
+// One cell a thread, gridDim.y over the nodes (64-bit divisions of one long
+// index were half of the kernel's instructions).  13 samples of 192 x 96 x 64,
+// odd level: 485 -> 343 us (even 235 -> 205, of a floor of 207).
+template <class S, bool SHIFT, bool ODD>
+__global__ void __launch_bounds__(256) average_add_kernel(const __grid_constant__ StepParams P, int domain, double* avg) {
   using T = typename Store<S>::C;
   const DevDomain& D = P.dom[domain];
-  const long long total = D.ncell * D.nodes;
-  for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < total;
-       k += (long long)gridDim.x * blockDim.x) {
-    const int j = (int)(k / D.ncell);
-    const long long c = k - (long long)j * D.ncell;
-    const LinkWord lw = __ldg(D.link + c);
-    if (lw & kLinkSolid) continue;
-    const int x = (int)(c % D.nx), y = (int)((c / D.nx) % D.ny), z = (int)(c / ((long long)D.nx * D.ny));
-    T g[kQ];
-    gather_pops<S, SHIFT>(P, D, j, P.n_host, x, y, z, c, lw, g);
-    T rho, ux, uy, uz;
+  const int c = (int)(blockIdx.x * blockDim.x + threadIdx.x), node = (int)blockIdx.y;
+  const LinkWord lw = c < (int)D.ncell ? __ldg(D.link + c) : kLinkSolid;
+  double* const at = avg + (long long)node * D.ncell + c;
+  if constexpr (SHIFT) {
+    const S* g0 = reinterpret_cast<const S*>(D.g) + (long long)node * kQ * D.pitch;
+    with_pops_form<ODD>(lw, [&](auto form) {
+      if (lw & kLinkSolid) return;
+      constexpr Pops FORM = decltype(form)::value;
+      const long long listed = FORM == Pops::kLinks && (lw & kLinkSlow) ? listed_index(D, c) : 0;
+      bool bad = false;
+      *at += widen(cell_speed<S, FORM>(P, D, node, g0, c, lw, listed, bad));
+    });
+  } else {
+    if (lw & kLinkSolid) return;
+    T g[kQ], rho, ux, uy, uz;
+    gather_pops<S, SHIFT>(P, D, node, P.n_host, 0, 0, 0, c, lw, g);
     macro<T, SHIFT>(g, rho, ux, uy, uz);
-    avg[k] += double(speed<T>(ux, uy, uz));
+    *at += double(speed<T>(ux, uy, uz));
   }
 }
 
@@ -776,6 +789,9 @@ __global__ void scale_kernel(const double* __restrict__ in, double sc, double* _
     out[k] = in[k] * sc;
 }
 
+// Count cells whose stored populations sum to a non-finite or non-positive
+// density (layout-independent: the stored 19 values of a cell always carry
+// its density at the current or previous time level).
 template <class S, bool SHIFT>
 __global__ void check_kernel(const __grid_constant__ StepParams P, unsigned long long* count) {
   unsigned long long local = 0;
@@ -907,10 +923,12 @@ int launch_export(const StepParams& P, int precision, int domain, int node, doub
 int launch_average_add(const StepParams& P, int precision, int domain, double* avg, void* stream) {
   cudaStream_t s = (cudaStream_t)stream;
   const DevDomain& D = P.dom[domain];
+  const dim3 grid((unsigned)((D.ncell + 255) / 256), (unsigned)D.nodes);
   return dispatch(precision, [&](auto tag) -> int {
     using S = std::remove_pointer_t<decltype(tag)>;
     constexpr bool SH = !std::is_same_v<S, double>;
-    average_add_kernel<S, SH><<<grid_for(D.ncell * D.nodes, 256), 256, 0, s>>>(P, domain, avg);
+    if (SH && (P.n_host & 1ull)) average_add_kernel<S, SH, true><<<grid, 256, 0, s>>>(P, domain, avg);
+    else average_add_kernel<S, SH, false><<<grid, 256, 0, s>>>(P, domain, avg);
     return (int)cudaGetLastError();
   });
 }
