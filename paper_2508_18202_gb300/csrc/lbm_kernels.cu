@@ -890,7 +890,7 @@ __global__ void __launch_bounds__(256, 3) aa_persistent_kernel(const __grid_cons
 // only the warps that have a moving-wall or specular link carry its FP64
 // terms.  The trailing blocks take the listed cells.  5 nodes of 48 x 24 x 24,
 // a time step: 400 us as one launch a node of 64 x 2 x 8 tiles (41 blocks on
-// 152 SMs), 59.5 us (FP64 pipe 81% busy); 2 of 128 x 64 x 48: 581 -> 370 us.
+// 152 SMs), 55.5 us; 2 of 128 x 64 x 48: 581 -> 318 us.
 constexpr int kPlainThreads = 128;
 
 __device__ __forceinline__ Node<double> plain_node(const DevDomain& D, double* dst, int node) {
