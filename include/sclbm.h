@@ -185,8 +185,9 @@ typedef struct {
  * packed FP32x2 operations; the block then covers 2 * block_x cells in x),
  * sized for 2 (variant 0) or 3 (variant 3) resident blocks; the results
  * equal the one-cell form's to FP32 rounding, not bit for bit.  Default:
- * launch mode, tile order 1, variant 0, block and slab by the ensemble's size
- * and collision (sc_lbm_get_tuning names them).                             */
+ * tile order 1, variant 0, block, slab and mode (launch, or graph for the
+ * smallest ensembles) by the ensemble's size and collision; sc_lbm_get_tuning
+ * names them.                                                               */
 typedef struct {
   int block_x, block_y, slab_z, tile_order, exec_mode, graph_steps, variant;
 } sc_lbm_tuning;
