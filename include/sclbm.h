@@ -183,7 +183,7 @@ typedef struct {
  * in every domain, variants 0 and 3 run the even level with two x-adjacent
  * cells per thread (one 32-bit access per population pair, the collision on
  * packed FP32x2 operations; the block then covers 2 * block_x cells in x),
- * sized for 2 (variant 0) or 3 (variant 3) resident blocks; the results
+ * sized for 3 resident blocks; the results
  * equal the one-cell form's to FP32 rounding, not bit for bit.  Default:
  * tile order 1, variant 0, block, slab and mode (launch, or graph for the
  * smallest ensembles) by the ensemble's size and collision; sc_lbm_get_tuning

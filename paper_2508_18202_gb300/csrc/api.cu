@@ -398,9 +398,8 @@ void apply_tiling(sc_lbm_t h) {
   P.odd85 = (h->tune.variant == 2 || h->tune.variant == 3) ? 1 : 0;
   // 16-bit storage with the BGK collision, every domain's rows pairing up
   // (even nx): two x-adjacent cells per thread on the even level in variants
-  // 0 (kernel sized for 2 resident blocks) and 3 (3 blocks)
-  const bool pairs = pairs_ok(h) && !P.tma;
-  P.even_pair = !pairs ? 0 : h->tune.variant == 0 ? 2 : h->tune.variant == 3 ? 3 : 0;
+  // 0 and 3
+  P.even_pair = pairs_ok(h) && !P.tma && (h->tune.variant == 0 || h->tune.variant == 3);
   if (h->graph) {
     cudaGraphExecDestroy(h->graph);
     h->graph = nullptr;

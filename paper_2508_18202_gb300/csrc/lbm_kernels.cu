@@ -476,11 +476,13 @@ __device__ __forceinline__ void even_run_pair(const StepParams& P, S* base, cons
 
 // Even time level with 16-bit storage, two cells per thread (launched with
 // the tiling of pair_tiling: tiles 2 * blockDim.x cells wide); the listed
-// cells ride in blocks spread over the grid as in aa_even_kernel.  MINB:
-// resident blocks of 256 threads (2: no spills at 110 registers; 3: 80
-// registers, a few bytes spilled, half as many warps again in flight).
-template <class S, int MINB>
-__global__ void __launch_bounds__(256, MINB) aa_even_pair_kernel(const __grid_constant__ StepParams P) {
+// cells ride in blocks spread over the grid as in aa_even_kernel.  Sized for 3
+// resident blocks of 256 threads (80 registers): the level waits on memory, and
+// half as many warps again in flight beat the 110 registers of 2 blocks (13
+// samples of 256 x 128 x 64, BF16: 394 against 441 us at 32 x 2 x 4; with the next
+// pair's words loaded ahead, 120 registers and 2 blocks, 412).
+template <class S>
+__global__ void __launch_bounds__(256, 3) aa_even_pair_kernel(const __grid_constant__ StepParams P) {
   unsigned k;
   if (block_role(P, &k)) {
     const long long item = k * (long long)(blockDim.x * blockDim.y) + threadIdx.y * blockDim.x + threadIdx.x;
@@ -1051,8 +1053,7 @@ int launch_aa_step(const StepParams& P, int precision, void* stream, int parity)
           if (P.even_pair && !P.tma) {
             unsigned qgrid = 0;
             const StepParams Q = with_listed_blocks(pair_tiling(P), threads, &qgrid);
-            if (P.even_pair == 3) aa_even_pair_kernel<S, 3><<<qgrid, block, 0, s>>>(Q);
-            else aa_even_pair_kernel<S, 2><<<qgrid, block, 0, s>>>(Q);
+            aa_even_pair_kernel<S><<<qgrid, block, 0, s>>>(Q);
             return (int)cudaGetLastError();
           }
         }
