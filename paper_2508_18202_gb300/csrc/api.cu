@@ -945,6 +945,10 @@ int sc_lbm_step(sc_lbm_t h, int n_steps) {
   return do_steps(h, n_steps);
 }
 
+// 1 / w for the kernels' quotients, or 0 (they divide) where w is too near the
+// ends of the range for the quotient's residual.
+static double reciprocal(double w) { return w > 1e-200 && w < 1e200 ? 1.0 / w : 0.0; }
+
 int sc_lbm_moments(sc_lbm_t h, int domain, double* mean, double* stdev, const int32_t* probe_xy,
                    int n_p, double* prof, float* prof_nodes, double* gpc_coef, int out_host) {
   if (!h || domain < 0 || domain >= h->P.n_domains) return SC_ERR_ARG;
@@ -966,7 +970,7 @@ int sc_lbm_moments(sc_lbm_t h, int domain, double* mean, double* stdev, const in
   A.stride = h->gpcP + 1;
   A.P = gpc_coef ? h->gpcP : 0;
   A.wsum = h->wsum[domain];
-  A.rwsum = 1.0 / A.wsum;
+  A.rwsum = reciprocal(A.wsum);
   A.mean = out_host ? (mean ? (double*)(h->ws + L.st_mean) : nullptr) : mean;
   A.stdev = out_host ? (stdev ? (double*)(h->ws + L.st_std) : nullptr) : stdev;
   A.coef = out_host ? (gpc_coef ? (double*)(h->ws + L.st_coef) : nullptr) : gpc_coef;
@@ -1016,7 +1020,7 @@ int sc_lbm_moment_sums(sc_lbm_t h, int domain, double* d_s1, double* d_s2, doubl
   A.stride = h->gpcP + 1;
   A.P = d_gpc_sums ? h->gpcP : 0;
   A.wsum = h->wsum[domain];
-  A.rwsum = 1.0 / A.wsum;
+  A.rwsum = reciprocal(A.wsum);
   A.mean = d_s1;
   A.stdev = d_s2;
   A.coef = d_gpc_sums;
@@ -1056,7 +1060,7 @@ int sc_lbm_moments_from_sums(sc_lbm_t h, int domain, const double* d_s1, const d
                              double* d_mean, double* d_stdev) {
   if (!h || !d_s1 || !d_s2 || !d_mean || !d_stdev || domain < 0 || domain >= h->P.n_domains) return SC_ERR_ARG;
   if (!(wsum > 0.0)) return fail(h, SC_ERR_ARG, "weight sum must be positive");
-  int rc = launch_finalize_moments(d_s1, d_s2, wsum, d_mean, d_stdev, h->P.dom[domain].ncell, h->stream);
+  int rc = launch_finalize_moments(d_s1, d_s2, wsum, reciprocal(wsum), d_mean, d_stdev, h->P.dom[domain].ncell, h->stream);
   if (rc) return cuda_fail(h, (cudaError_t)rc, "finalize launch");
   ++h->launches;
   return SC_OK;

@@ -133,7 +133,9 @@ __device__ __forceinline__ double widen(float v) {
 
 // a / w with r = 1 / w correctly rounded, itself correctly rounded (as
 // quotient() above): three FP64 instructions instead of a division's dozen.
+// r = 0: no such reciprocal, divide.
 __device__ __forceinline__ double quotient(double a, double w, double r) {
+  if (__double2hiint(r) == 0) return __ddiv_rn(a, w);
   const double q = __dmul_rn(a, r);
   if (((uint32_t)__double2hiint(q) & 0x7ff00000u) == 0x7ff00000u) return q;  // infinite or NaN: no residual
   return __fma_rn(__fma_rn(-w, q, a), r, q);
@@ -354,7 +356,9 @@ __device__ __forceinline__ void with_pops_form(LinkWord lw, F&& f) {
 // agrees with one reduction over all nodes to the pairs' 48-bit rounding.
 // This form serves the small bases (PM <= kMomCellMaxP); a large basis holds
 // too many accumulators per thread for it and goes to moments_split_kernel.
-// Up to 10 terms three blocks are resident per SM (80 registers).
+// Up to 10 terms three blocks are resident per SM (80 registers); four at 10
+// terms and an even level, which holds no links (2.43 -> 2.30 ms on 6 samples of
+// 512 x 256 x 128; no gain below).
 // Bound: the FP64 pipe where the nodes are few (16 cycles of an SM for an
 // instruction of a warp), so conversions go by the bits, the sums are only
 // converted where they continue, and a mean divides by a reciprocal; else the
@@ -364,7 +368,7 @@ __device__ __forceinline__ void with_pops_form(LinkWord lw, F&& f) {
 constexpr int kMomCellMaxP = 12;
 
 template <class S, int PM, bool ODD>
-__global__ void __launch_bounds__(256, PM <= 10 ? 3 : 2) moments_pair_kernel(const __grid_constant__ StepParams P, MomentArgs A) {
+__global__ void __launch_bounds__(256, !ODD && PM == 10 ? 4 : PM <= 10 ? 3 : 2) moments_pair_kernel(const __grid_constant__ StepParams P, MomentArgs A) {
   constexpr int NP = PM > 0 ? PM / 2 : 1;
   const DevDomain& D = P.dom[A.domain];
   const int c = (int)(blockIdx.x * blockDim.x + threadIdx.x);  // 19 ncell < 2^31
@@ -439,15 +443,15 @@ __global__ void __launch_bounds__(256, PM <= 10 ? 3 : 2) moments_pair_kernel(con
 // the accumulators.  PM = gpc_pair_pad(A.P) is the padded basis size (a
 // multiple of 4) and the row length of A.abf; its pad terms are zero and are
 // not written.  raw and accumulate as in moments_pair_kernel; the two forms
-// give the same bits (measured on 6-, 10- and 21-term bases).  121 samples of
-// 96 x 96 x 40, 21 terms, even / odd level: 1.23 / 1.61 -> 0.98 / 1.27 ms.  Three blocks per SM (80 registers, a few bytes
-// spilled at the largest bases) beat two unspilled ones: the wait on
-// dependent loads and arithmetic, not the instruction count, bounds this
-// reduction.
+// give the same bits (measured on 6-, 10- and 21-term bases).  Bound: the wait
+// on dependent loads and arithmetic, so warps in flight count for more than
+// spills of a few bytes: four blocks per SM at even levels, three at odd ones
+// (80 registers; two are 1.21 against 0.98 ms at an even level).  121 samples of
+// 96 x 96 x 40, 21 terms, even / odd level: 1.23 / 1.61 -> 0.93 / 1.27 ms.
 constexpr int kMomPairs = 4;  // warp pairs per block (256 threads, 128 cells)
 
 template <class S, int PM, bool ODD>
-__global__ void __launch_bounds__(64 * kMomPairs, 3) moments_split_kernel(const __grid_constant__ StepParams P,
+__global__ void __launch_bounds__(64 * kMomPairs, ODD ? 3 : 4) moments_split_kernel(const __grid_constant__ StepParams P,
                                                                          MomentArgs A) {
   static_assert(PM % 4 == 0, "two packed pairs of terms per thread pair");
   constexpr int NH = PM > 0 ? PM / 4 : 1;  // packed pairs per thread
@@ -933,9 +937,10 @@ int launch_average_add(const StepParams& P, int precision, int domain, double* a
   });
 }
 
-int launch_finalize_moments(const double* s1, const double* s2, double wsum, double* mean, double* stdev,
-                            long long n, void* stream) {
-  finalize_moments_kernel<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(s1, s2, wsum, 1.0 / wsum, mean, stdev, n);
+int launch_finalize_moments(const double* s1, const double* s2, double wsum, double rwsum, double* mean,
+                            double* stdev, long long n, void* stream) {
+  finalize_moments_kernel<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(s1, s2, wsum, rwsum, mean,
+                                                                                  stdev, n);
   return (int)cudaGetLastError();
 }
 

@@ -246,7 +246,7 @@ struct MomentArgs {
                            // (hi_a, hi_a+1, lo_a, lo_a+1) floats, hi + lo to 48 bits; zero pad terms
   int stride;              // row length of ab (basis size of the configuration + 1)
   int nq, P;               // P: coefficients to produce (0 = none)
-  double wsum, rwsum;      // sum of the weights, and 1 / wsum correctly rounded
+  double wsum, rwsum;      // sum of the weights, and 1 / wsum correctly rounded (0: divide by wsum)
   double* mean;
   double* stdev;
   double* coef;            // [P][ncell] or null
@@ -265,8 +265,9 @@ int launch_export(const StepParams& P, int precision, int domain, int node, doub
 // Adds |u| of every node of a domain at the current time level to avg[nq][ncell].
 int launch_average_add(const StepParams& P, int precision, int domain, double* avg, void* stream);
 // mean = s1 / wsum, stdev = sqrt(max(s2 / wsum - mean^2, 0)), n cells.
-int launch_finalize_moments(const double* s1, const double* s2, double wsum, double* mean, double* stdev,
-                            long long n, void* stream);
+// rwsum: as in MomentArgs.
+int launch_finalize_moments(const double* s1, const double* s2, double wsum, double rwsum, double* mean,
+                            double* stdev, long long n, void* stream);
 // out[k] = s * in[k], k < n.
 int launch_scale(const double* in, double s, double* out, long long n, void* stream);
 // Q-criterion of a velocity field u[3][ncell] of a domain into q[ncell].
