@@ -328,6 +328,7 @@ struct sc_lbm_s {
   int persist_grid = 0;
   int never_arrive = 0;
   long long spin_limit = kSpinLimit;
+  bool shape_given = false;  // the launch shape was set or tuned, not the default
   int tma_ok = 0;  // every domain's rows meet the 16-byte alignment of bulk copies
   Header* hdr() const { return reinterpret_cast<Header*>(ws + L.hdr); }
 };
@@ -627,7 +628,10 @@ int run_aa(sc_lbm_t h, int n) {
       n -= 1;
     } else {
       const Wind<double> w = wind_at(h, t);
-      if (h->tune.exec_mode == SC_EXEC_GRAPH) rc = run_graph(h, t, (int)c, w);
+      // the default mode takes no graphs under a series: each hold has a
+      // factor of its own, and a capture costs more than the hold's launches
+      const bool graphs = h->tune.exec_mode == SC_EXEC_GRAPH && (h->shape_given || h->series_speed.empty());
+      if (graphs) rc = run_graph(h, t, (int)c, w);
       else if (h->tune.exec_mode == SC_EXEC_PERSISTENT) rc = run_persistent(h, t, (int)c, w);
       else rc = run_launches(h, t, (int)c);
       t += c;
@@ -1192,6 +1196,7 @@ int sc_lbm_set_tuning(sc_lbm_t h, const sc_lbm_tuning* t) {
   if (!h || !t || check_tuning(*t)) return SC_ERR_ARG;
   CK(cudaStreamSynchronize(h->stream));
   h->tune = *t;
+  h->shape_given = true;
   apply_tiling(h);
   return SC_OK;
 }
