@@ -20,7 +20,7 @@ roofline   the stream-collide kernels: algorithmic bytes (152 B per fluid
            cell update in FP32, 19 reads + 19 writes) per time step over the
            average time-step duration (CUDA events on the library's stream),
            against the measured HBM copy bandwidth.
-Extra keys: the plain one-node-at-a-time FP64 GPU path on the same domain,
+Extra keys: the plain FP64 GPU path on the same domain,
 the 256x128x64 13-node LES ensemble and the three-domain batched ensemble
 (FP32 and BF16 storage, autotuned) with the error of their mean / std fields
 against the FP64 path, BF16 / FP16 storage, the paper's collision, an hourly
@@ -355,9 +355,8 @@ def field_errors(cx, wl, precisions, steps, ramp):
 
 
 def leg_plain(cx, wl, glups):
-    """Plain FP64, one node per launch, on the headline domain: two nodes of
-    the rule (the path runs nodes one after another, so GLUPS per node is the
-    ensemble's)."""
+    """Plain FP64 on the headline domain: two nodes of the rule (the FP64 pipe
+    bounds the path, so their GLUPS is the ensemble's)."""
     S, W = cx.S, cx.W
     nodes = 2
     pw = dict(wl, precision=W.FP64_PLAIN, node_begin=0, node_count=nodes)
