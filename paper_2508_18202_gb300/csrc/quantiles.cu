@@ -277,7 +277,12 @@ int launch_group(const double* coef, long long ncell, int P, const int32_t* cell
                  const float* phif, int M, int Mf, int Mp, const BasisBound& bound, const int32_t* kidx, int nq,
                  double* out, cudaStream_t s) {
   const size_t smem = std::max(sizeof(float) * (size_t)G * Mf, sizeof(double) * (size_t)Mp);
-  cudaError_t e = cudaFuncSetAttribute(gpc_quantile_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the same limit from every call, so that calls from several threads do not
+  // lower one another's
+  constexpr int kMostValues = 4 * 8 * 4096;
+  static_assert(4 * 4 * SC_QUANTILE_MAX_SAMPLES <= kMostValues && 8 * SC_QUANTILE_MAX_SAMPLES <= kMostValues,
+                "four cells' FP32 values and one cell's FP64 values fit");
+  cudaError_t e = cudaFuncSetAttribute(gpc_quantile_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMostValues);
   if (e != cudaSuccess) return (int)e;
   gpc_quantile_kernel<G><<<(n_cells + G - 1) / G, kThreads, smem, s>>>(coef, ncell, P, cells, n_cells, phi, phif, M,
                                                                        Mf, Mp, bound, kidx, nq, out);
