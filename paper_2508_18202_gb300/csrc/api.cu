@@ -516,13 +516,51 @@ int run_launches(sc_lbm_t h, long long start, int n) {
   return SC_OK;
 }
 
+// Puts the calling thread's capture mode to relaxed while it lives: calls that
+// a capture of another of the caller's streams would refuse (and be broken by)
+// are made here on a stream of the library's own.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// The graph of G levels from an even one under the factor w.  It is recorded
+// on a stream of its own, which nothing else launches into: the handle's
+// stream may be a blocking one, whose capture a legacy-stream call of any
+// thread breaks, or one that another thread's handle launches into as well,
+// whose kernels the capture would take in.
+cudaError_t record_levels(sc_lbm_t h, int G, const Wind<double>& w, cudaGraphExec_t* out) {
+  RelaxedCapture relaxed;
+  cudaStream_t s = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return e;
+  cudaGraph_t g = nullptr;
+  e = cudaStreamBeginCapture(s, cudaStreamCaptureModeRelaxed);
+  if (e == cudaSuccess) {
+    int rc = 0;
+    StepParams P = h->P;
+    set_winds(P, w);
+    for (int k = 0; k < G && !rc; ++k)
+      rc = h->cfg.collision == SC_COLL_RR ? rr::launch_aa_step(P, h->cfg.precision, s, k & 1)
+                                          : launch_aa_step(P, h->cfg.precision, s, k & 1);
+    e = cudaStreamEndCapture(s, &g);
+    if (rc) e = (cudaError_t)rc;
+  }
+  if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
+  if (g) cudaGraphDestroy(g);
+  cudaStreamDestroy(s);
+  return e;
+}
+
 // Replays of a captured graph of G steps (even/odd pairs, G even) starting
 // at an even time level, over levels [t, t + n) of constant inflow factor w.
 // The graph holds w in its launch parameters; it is captured again when a
 // stretch with another factor comes.
 int run_graph(sc_lbm_t h, long long t, int n, const Wind<double>& w) {
   const int G = h->tune.graph_steps + (h->tune.graph_steps & 1);
-  if (!h->stream) return run_launches(h, t, n);  // capture needs a non-default stream
+  // the legacy default stream, under either of its names, takes launches
+  if (!h->stream || h->stream == cudaStreamLegacy) return run_launches(h, t, n);
   // a caller capturing the stream records the levels' kernels
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
   CK(cudaStreamIsCapturing(h->stream, &capturing));
@@ -542,23 +580,15 @@ int run_graph(sc_lbm_t h, long long t, int n, const Wind<double>& w) {
     if (h->graph) cudaGraphExecDestroy(h->graph);
     h->graph = nullptr;
     h->graph_len = 0;
-    cudaGraph_t g = nullptr;
-    CK(cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-    int rc = 0;
-    StepParams P = h->P;
-    set_winds(P, w);
-    for (int s = 0; s < G && !rc; ++s)
-      rc = h->cfg.collision == SC_COLL_RR ? rr::launch_aa_step(P, h->cfg.precision, h->stream, s & 1)
-                                          : launch_aa_step(P, h->cfg.precision, h->stream, s & 1);
-    cudaError_t e = cudaStreamEndCapture(h->stream, &g);
-    if (rc) {
-      if (g) cudaGraphDestroy(g);
-      return cuda_fail(h, (cudaError_t)rc, "graph capture launch");
+    const cudaError_t e = record_levels(h, G, w, &h->graph);
+    if (e != cudaSuccess) {
+      h->graph = nullptr;
+      if (h->shape_given) return cuda_fail(h, e, "graph of the levels");
+      // the default mode was not the caller's choice: launches from here on
+      cudaGetLastError();
+      h->tune.exec_mode = SC_EXEC_LAUNCH;
+      return run_launches(h, t, n);
     }
-    if (e != cudaSuccess) return cuda_fail(h, e, "cudaStreamEndCapture");
-    e = cudaGraphInstantiate(&h->graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return cuda_fail(h, e, "cudaGraphInstantiate");
     h->graph_len = G;
     h->graph_wind = wf;
   }

@@ -1,0 +1,133 @@
+"""Handles of the smallest ensembles, whose default mode replays captured
+graphs, on the streams and beside the threads that a handle stepped by
+launches can be used with."""
+import threading
+
+import numpy as np
+import pytest
+
+from paper_2508_18202_gb300 import sclbm as S
+from paper_2508_18202_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+WL = dict(domains=[dict(nx=45, ny=21, nz=14, boxes=[[8, 4, 0, 13, 10, 6]], bc=W.URBAN_BC, quad_level=3)], tau0=0.52,
+          c_smag=0.14, u_ref=0.05, alpha=0.25, angle_deg=5.0, H_ref=0.0, inputs=[W.SPEED], lo=[-0.1], hi=[0.1],
+          quad_rule=W.GL, ramp_steps=0, precision=W.FP32_SHIFT, gpc_degree=2)
+LEGACY, PER_THREAD = 1, 2   # the runtime's names of the default streams
+
+
+class Handle:
+    """A handle at its default shape on a raw stream."""
+
+    def __init__(self, stream, launches=False):
+        self.cfg = S.make_config(WL)
+        n = S.sc_lbm_workspace_size(self.cfg)
+        self.ws = torch.empty(n, dtype=torch.uint8, device="cuda")
+        self.f = torch.empty(19, 45 * 21 * 14, dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        self.h = S.sc_lbm_init(self.cfg, self.ws.data_ptr(), n, stream)
+        t = S.sc_lbm_get_tuning(self.h)
+        assert t["exec_mode"] == S.SC_EXEC_GRAPH
+        if launches:
+            S.sc_lbm_set_tuning(self.h, **dict(t, exec_mode=S.SC_EXEC_LAUNCH))
+
+    def step(self, n):
+        S.sc_lbm_step(self.h, n)
+
+    def state(self):
+        S.sc_lbm_populations(self.h, 0, 1, self.f)
+        S.sc_lbm_sync(self.h)
+        return self.f.cpu().numpy()
+
+    def close(self):
+        S.sc_lbm_destroy(self.h)
+
+
+@pytest.fixture(scope="module")
+def want():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    ref = Handle(torch.cuda.Stream().cuda_stream, launches=True)
+    ref.step(41)
+    out = ref.state()
+    ref.close()
+    return out
+
+
+@pytest.mark.parametrize("stream", [0, LEGACY, PER_THREAD])
+def test_default_streams(want, stream):
+    h = Handle(stream)
+    for n in (25, 16):
+        h.step(n)
+    assert np.array_equal(h.state(), want)
+    h.close()
+
+
+@pytest.mark.parametrize("blocking", [False, True])
+def test_another_thread_uses_the_stream_and_the_legacy_one(want, blocking):
+    """New handles step (and capture) while another thread launches into their
+    stream and into the legacy stream, and while it steps a handle of its own
+    on the same stream: each handle's levels are its own."""
+    cudart = torch.cuda.cudart()
+    own = torch.cuda.Stream()
+    raw = own.cuda_stream
+    if blocking:
+        raw_p = torch.zeros(1, dtype=torch.int64)
+        assert int(cudart.cudaStreamCreate(raw_p.data_ptr())) == 0
+        raw = int(raw_p[0])
+    shared = torch.cuda.ExternalStream(raw)
+    other = Handle(raw, launches=True)
+    stop, errors, levels = threading.Event(), [], [0]
+    x, y = torch.zeros(1024, device="cuda"), torch.zeros(1024, device="cuda")
+    torch.cuda.synchronize()
+
+    def work():
+        try:
+            while not stop.is_set():
+                x.add_(1.0)
+                with torch.cuda.stream(shared):
+                    y.add_(1.0)
+                if levels[0] < 41:
+                    other.step(1)
+                    levels[0] += 1
+        except Exception as e:   # reported by the main thread
+            errors.append(e)
+
+    t = threading.Thread(target=work)
+    t.start()
+    try:
+        for _ in range(20):
+            h = Handle(raw)
+            h.step(41)
+            assert np.array_equal(h.state(), want)
+            h.close()
+    finally:
+        stop.set()
+        t.join()
+    assert not errors, errors
+    other.step(41 - levels[0])
+    assert np.array_equal(other.state(), want)
+    other.close()
+    torch.cuda.synchronize()
+    if blocking:
+        assert int(cudart.cudaStreamDestroy(raw)) == 0
+
+
+def test_while_the_caller_records_another_stream(want):
+    """A handle steps for the first time while its thread records a graph on
+    another stream; that record stays whole."""
+    h = Handle(torch.cuda.Stream().cuda_stream)
+    x = torch.zeros(64, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g):
+        x.add_(1.0)
+        h.step(41)
+        x.add_(1.0)
+    g.replay()
+    torch.cuda.synchronize()
+    assert float(x[0]) == 2.0
+    assert np.array_equal(h.state(), want)
+    h.close()
