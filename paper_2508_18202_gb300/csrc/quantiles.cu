@@ -98,8 +98,10 @@ __global__ void __launch_bounds__(kThreads) gpc_quantile_kernel(
   // max |Phi_a| a rounding of the coefficient, one of the basis value and P of
   // the sum make at most (P + 2) 2^-24 S (1 + O(2^-24)); twice that is taken.
   // 0 for a cell without coefficients, +inf where a float does not carry a
-  // factor or S (a coefficient or basis bound outside 1e-30 .. 1e30, S outside
-  // 1e-20 .. 1e25), or one is not a number.  In FP32, one warp a cell: in FP64
+  // factor or S (a coefficient or its basis bound outside 1e-30 .. 1e30, S
+  // outside 1e-20 .. 1e25), or one is not a number.  A basis bound from 1e30 on
+  // counts without a coefficient as well: the basis value may be infinite as a
+  // float, and zero times it is no number.  In FP32, one warp a cell: in FP64
   // by every thread it was half of the kernel.
   for (int g = threadIdx.x / 32; g < G; g += kThreads / 32) {
     const int a = threadIdx.x % 32;
@@ -107,15 +109,15 @@ __global__ void __launch_bounds__(kThreads) gpc_quantile_kernel(
     const bool some = (__double_as_longlong(c) << 1) != 0;
     const float f = fabsf((float)c), m = a < P ? bound.m[a] : 1.0f;
     float S = some ? f * m : 0.0f, v2 = a > 0 ? f * f : 0.0f;
-    const bool off = some && !(f > 1e-30f && f < 1e30f && m > 1e-30f && m < 1e30f);
+    const bool off = !(m < 1e30f) || (some && !(f > 1e-30f && f < 1e30f && m > 1e-30f));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       S += __shfl_xor_sync(0xffffffffu, S, o);
       v2 += __shfl_xor_sync(0xffffffffu, v2, o);
     }
-    const bool any = __any_sync(0xffffffffu, some), bad = __any_sync(0xffffffffu, off) || !(S > 1e-20f && S < 1e25f);
+    const bool any = __any_sync(0xffffffffu, some), bad = __any_sync(0xffffffffu, off);
     if (a == 0) {
-      err[g] = !any ? 0.0f : bad ? INFINITY : S * (float)(P + 4) * 1.1920929e-7f;
+      err[g] = bad ? INFINITY : !any ? 0.0f : S > 1e-20f && S < 1e25f ? S * (float)(P + 4) * 1.1920929e-7f : INFINITY;
       mid[g] = (float)c;
       spread[g] = 5.0f * sqrtf(v2);
     }
