@@ -247,29 +247,29 @@ __global__ void __launch_bounds__(kThreads) gpc_quantile_kernel(
   }
   if (t == 0) whole[g] = mine && sort;
   __syncthreads();
-  // cells left whole: all M values in FP64, sorted ascending with a bitonic
-  // network (the tail padded with +inf)
+  // cells left whole: all M values in FP64, as integers of their order sorted
+  // ascending with a bitonic network over Mp >= M (a power of two) of them, the
+  // tail padded with the largest one
+  long long* const keys = reinterpret_cast<long long*>(values);
   for (int h = 0; h < G; ++h) {
     if (!whole[h]) continue;
     for (int m = threadIdx.x; m < Mp; m += kThreads)
-      values[m] = m < M ? surrogate(phi + (long long)m * P, cs[h], P) : INFINITY;
+      keys[m] = m < M ? ordered(surrogate(phi + (long long)m * P, cs[h], P)) : 0x7fffffffffffffffLL;
     __syncthreads();
     for (int k = 2; k <= Mp; k <<= 1)
       for (int j = k >> 1; j > 0; j >>= 1) {
-        for (int i = threadIdx.x; i < Mp; i += kThreads) {
-          const int l = i ^ j;
-          if (l > i) {
-            const double a = values[i], b = values[l];
-            const bool up = (i & k) == 0;
-            if (up ? (a > b) : (a < b)) {
-              values[i] = b;
-              values[l] = a;
-            }
+        for (int p = threadIdx.x; p < Mp / 2; p += kThreads) {  // the pairs (i, i + j)
+          const int i = 2 * p - (p & (j - 1)), l = i + j;
+          const long long a = keys[i], b = keys[l];
+          if ((a > b) == ((i & k) == 0)) {
+            keys[i] = b;
+            keys[l] = a;
           }
         }
         __syncthreads();
       }
-    for (int j = threadIdx.x; j < nq; j += kThreads) out[(long long)j * n_cells + cell0 + h] = values[kidx[j] - 1];
+    for (int j = threadIdx.x; j < nq; j += kThreads)
+      out[(long long)j * n_cells + cell0 + h] = from_ordered(keys[kidx[j] - 1]);
     __syncthreads();
   }
 }
