@@ -1125,15 +1125,12 @@ int sc_lbm_gpc_quantiles(sc_lbm_t h, int domain, const double* d_coef, int n_cel
                  h->cfg.quad_rule == SC_Q_GH);
   }
   if (n_cells == 0) return SC_OK;
-  double phi_max[kMaxGpcP] = {}, phi_sum[kMaxGpcP] = {};
+  // A NaN passes the maximum by, but its term is not alone: a recurrence gives
+  // one only after an infinite value of a lower order, whose own term is infinite
+  // for the same sample.
+  double phi_max[kMaxGpcP] = {};
   for (int m = 0; m < n_samples; ++m)
-    for (int a = 0; a < P; ++a) {
-      const double v = std::fabs(phi[(size_t)m * P + a]);
-      phi_max[a] = std::max(phi_max[a], v);
-      phi_sum[a] += v;
-    }
-  for (int a = 0; a < P; ++a)  // a NaN is in the sum, not in the maximum
-    if (!std::isfinite(phi_sum[a])) phi_max[a] = INFINITY;
+    for (int a = 0; a < P; ++a) phi_max[a] = std::max(phi_max[a], std::fabs(phi[(size_t)m * P + a]));
   std::vector<int32_t> cl(cells, cells + n_cells);
   const Layout& L = h->L;
   // pageable sources: each copy has taken its data when the call returns

@@ -57,9 +57,10 @@ __device__ __forceinline__ double surrogate(const double* __restrict__ row, cons
 }
 
 // A double as a signed integer of the same order, and back (compared on the
-// integer pipe).
+// integer pipe); every NaN is the largest.
 __device__ __forceinline__ long long ordered(double v) {
   const long long b = __double_as_longlong(v);
+  if ((b & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL) return 0x7fffffffffffffffLL;
   return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
 }
 __device__ __forceinline__ double from_ordered(long long k) {

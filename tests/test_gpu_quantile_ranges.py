@@ -50,6 +50,32 @@ def test_basis_beyond_the_float_range(cuda, n_cells):
     ens.close()
 
 
+def test_basis_that_is_not_a_number(cuda):
+    """A sample so far out that the fourth-order basis value is inf - inf: the
+    surrogate is not a number there (the sorts place it last), and all other
+    ranks are those of the remaining samples, also where the infinite
+    second- and third-order terms have no coefficient."""
+    ens = ensemble(gpc_degree=4)
+    n = 16 * 16 * 8
+    rng = np.random.RandomState(1)
+    coef = np.zeros((5, n))
+    coef[0] = 1.0 + rng.rand(n)
+    coef[1] = 1e-3
+    coef[4, ::2] = 1e-4
+    samples = rng.uniform(-2.0, 2.0, (41, 1))
+    samples[5] = 1e200
+    with np.errstate(over="ignore", invalid="ignore"):
+        he4 = (samples ** 4 - 6.0 * samples ** 2 + 3.0) / np.sqrt(24.0)
+    rest = np.delete(np.arange(41), 5)
+    y = np.sort((coef[0] + samples * coef[1] + he4 * coef[4])[rest], axis=0)
+    cells = np.arange(n, dtype=np.int32)
+    q = np.arange(1, 41, 5) / 41.0
+    got = ens.gpc_quantiles(0, torch.from_numpy(coef).cuda(), cells, samples, list(q)).cpu().numpy()
+    ranks = [int(np.ceil(v * 41)) - 1 for v in q]
+    assert np.all(np.abs(got - y[ranks]) <= 64 * 2.0 ** -52 * 3.0)
+    ens.close()
+
+
 def hermite_basis(samples):
     """Orthonormal Hermite products of total degree <= 3 in two inputs."""
     he = [np.polynomial.hermite_e.hermeval(samples, [0] * k + [1]) / np.sqrt([1.0, 1.0, 2.0, 6.0][k]) for k in range(4)]
