@@ -685,13 +685,14 @@ __device__ __forceinline__ Diff two_diff(float a, float b) {
 }
 
 // Q of a cell whose gradient has entries near the end of the float range or
-// beyond it, in FP64: J = (up - dn) f, f the axis' factor.
+// beyond it, in FP64: J = (up - dn) f, f the axis' factor, and 0 whatever the
+// velocity is where the factor is 0 (an axis without a fluid neighbour).
 __device__ __noinline__ float qcriterion_wide(const float up[3][3], const float dn[3][3], const float f[3]) {
   double s2 = 0.0, w2 = 0.0;
   for (int i = 0; i < 3; ++i)
     for (int a = 0; a < 3; ++a) {
-      const double ja = (double)f[a] * ((double)up[i][a] - (double)dn[i][a]);
-      const double ji = (double)f[i] * ((double)up[a][i] - (double)dn[a][i]);
+      const double ja = f[a] == 0.0f ? 0.0 : (double)f[a] * ((double)up[i][a] - (double)dn[i][a]);
+      const double ji = f[i] == 0.0f ? 0.0 : (double)f[i] * ((double)up[a][i] - (double)dn[a][i]);
       const double sv = 0.5 * (ja + ji), wv = 0.5 * (ja - ji);
       s2 += sv * sv;
       w2 += wv * wv;
@@ -720,7 +721,7 @@ __global__ void __launch_bounds__(256) qcriterion_kernel(const __grid_constant__
     const int hi = last ? c - (dim[a] - 1) * step[a] : c + step[a];
     const bool ok0 = (!first || wrap) && !D.flags[lo], ok1 = (!last || wrap) && !D.flags[hi];
     const int c0 = ok0 ? lo : c, c1 = ok1 ? hi : c;
-    f[a] = ok0 && ok1 ? 0.5f : 1.0f;
+    f[a] = ok0 && ok1 ? 0.5f : ok0 || ok1 ? 1.0f : 0.0f;
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       up[i][a] = u[i * ncell + c1];
