@@ -78,10 +78,12 @@ __device__ __forceinline__ void gather_pops(const StepParams& P, const DevDomain
 // corrects it to the correctly rounded a / b (Markstein, "Computation of
 // elementary functions on the IBM RISC System/6000 processor", IBM J. Res.
 // Develop. 34, 1990), so three quotients by one density cost one reciprocal.
-// (Below 2^-102 the residual may be inexact and the last bit differ.)
+// The residual is taken negated: b q - a keeps a zero's sign through the
+// correction.  Finite a and q.  (Below 2^-102 the residual may be inexact and
+// the last bit differ.)
 __device__ __forceinline__ float quotient(float a, float b, float r) {
   const float q = __fmul_rn(a, r);
-  return __fmaf_rn(__fmaf_rn(-b, q, a), r, q);
+  return __fmaf_rn(-__fmaf_rn(b, q, -a), r, q);
 }
 
 // Density and velocity from the populations gather_pops gives (Sec. 2.2:
@@ -94,7 +96,9 @@ __device__ __forceinline__ void macro(const T g[kQ], T& rho, T& ux, T& uy, T& uz
   flow_sums<T>(g, m0, jx, jy, jz);
   rho = SHIFT ? T(1) + m0 : m0;
   if constexpr (sizeof(T) == 4) {
-    if (rho > 1e-18f && rho < 1e18f) {
+    // one bound for the density and the momentum: with it the quotients stay
+    // below 1e36, and a momentum that is infinite divides
+    if (rho > 1e-18f && (fabsf(jx) + fabsf(jy)) + (fabsf(jz) + rho) < 1e18f) {
       const float r = recip(rho);
       ux = quotient(jx, rho, r);
       uy = quotient(jy, rho, r);
@@ -138,7 +142,7 @@ __device__ __forceinline__ double quotient(double a, double w, double r) {
   if (__double2hiint(r) == 0) return __ddiv_rn(a, w);
   const double q = __dmul_rn(a, r);
   if (((uint32_t)__double2hiint(q) & 0x7ff00000u) == 0x7ff00000u) return q;  // infinite or NaN: no residual
-  return __fma_rn(__fma_rn(-w, q, a), r, q);
+  return __fma_rn(-__fma_rn(w, q, -a), r, q);
 }
 
 // mean = S1 / W, std = sqrt(max(S2 / W - mean^2, 0)) (Eq. quad_moments; the

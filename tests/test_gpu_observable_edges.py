@@ -42,3 +42,57 @@ def test_qcriterion_of_an_axis_without_fluid_neighbours(O, value):
     assert np.isfinite(want[corridor])
     assert abs(q[corridor] - want[corridor]) <= abs(want[corridor]) * 2.0 ** -24 + 36.0 * 2.0 ** -40
     ens.close()
+
+
+C_LAT = np.array([(0, 0, 0), (1, 0, 0), (-1, 0, 0), (0, 1, 0), (0, -1, 0), (0, 0, 1), (0, 0, -1), (1, 1, 0),
+                  (-1, -1, 0), (1, -1, 0), (-1, 1, 0), (1, 0, 1), (-1, 0, -1), (1, 0, -1), (-1, 0, 1), (0, 1, 1),
+                  (0, -1, -1), (0, 1, -1), (0, -1, 1)])
+
+
+def test_velocity_is_the_rounded_quotient():
+    """The exported velocity is momentum over density rounded once, bit for bit,
+    on random populations and on those of a zero of either sign, of an infinite
+    momentum at a finite density, and of a quotient beyond the float range."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    nx, ny, nz = 19, 7, 5
+    n, pitch, hdr = nx * ny * nz, 768, 48
+    ens = ensemble(nx, ny, nz)
+    buf = np.zeros(S.sc_lbm_state_size(ens.h), np.uint8)
+    S.sc_lbm_save(ens.h, buf)
+    g = buf[hdr:].view(np.float32)[19 * pitch:2 * 19 * pitch].reshape(19, pitch)   # node 1, level 0: natural order
+    rng = np.random.RandomState(4)
+    g[:, :n] = rng.uniform(-0.02, 0.02, (19, n))
+    g[:, :40] *= np.float32(1e-12)
+    for axis in range(3):
+        for sign in (1, -1):
+            c = 100 + 2 * axis + (sign < 0)
+            g[:, c] = np.where(C_LAT[:, axis] * sign > 0, np.float32(-0.0), np.float32(0.0))
+    g[:, 110:118] = 0.0
+    for k, (p, m) in enumerate([(1, 2), (2, 1), (3, 4), (5, 6)]):
+        g[p, 110 + k], g[m, 110 + k] = 3e38, -3e38                # infinite momentum, density 1
+        g[p, 114 + k], g[m, 114 + k] = 1e32, -1e32                # 2e32 over a density of 2^-24
+        g[18, 114 + k] = np.float32(2.0 ** -24 - 1.0)             # (added last, after the two cancel)
+    with np.errstate(over="ignore"):
+        m0, j = g[0, :n].copy(), [np.zeros(n, np.float32) for _ in range(3)]
+        for a in range(3):
+            j[a] = g[1 + 2 * a, :n].copy()
+        for i in range(1, 19):
+            m0 = m0 + g[i, :n]
+            for a in range(3):
+                if C_LAT[i, a] and i > 1 + 2 * a:
+                    j[a] = j[a] + np.float32(C_LAT[i, a]) * g[i, :n]
+        rho = np.float32(1.0) + m0
+        want = np.stack([j[a] / rho for a in range(3)])
+    assert np.all(rho > 0) and np.isinf(want[0, 110]) and np.isinf(want[0, 114])
+    assert np.signbit(want[0, 100]) and want[0, 100] == 0 and np.signbit(want[2, 104])
+    h = 1469598103934665603
+    for byte in buf[hdr:].tobytes():
+        h = ((h ^ byte) * 1099511628211) & ((1 << 64) - 1)
+    buf[24:32] = np.frombuffer(np.uint64(h).tobytes(), np.uint8)
+    S.sc_lbm_load(ens.h, buf)
+    got = ens.velocity(0, 1).cpu().numpy()
+    fluid = S.sc_lbm_geometry(ens.cfg, 0) == 0
+    assert fluid.all()
+    assert np.array_equal(got.view(np.int32), want.astype(np.float32).view(np.int32))
+    ens.close()
