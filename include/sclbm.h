@@ -359,7 +359,7 @@ int sc_lbm_qcriterion(sc_lbm_t h, int domain, const float* d_u, float* d_q);
 int sc_lbm_populations(sc_lbm_t h, int domain, int node, double* d_f);
 
 /* Launch shape: sc_lbm_autotune times candidate shapes on the current
- * configuration, keeps the fastest and resets the populations afterwards
+ * configuration, the handle's own among them, keeps the fastest and resets the populations afterwards
  * (tuning steps advance the state).  cache_path (host string, may be NULL)
  * names a JSON file whose entry for this GPU and configuration is reused or
  * written.  Synchronises.                                                   */

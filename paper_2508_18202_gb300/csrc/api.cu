@@ -1249,12 +1249,21 @@ int sc_lbm_autotune(sc_lbm_t h, const char* cache_path) {
   CK(cudaGetDevice(&dev));
   CK(cudaGetDeviceProperties(&prop, dev));
   const std::string key = tune_key(&h->cfg, prop.name);
+  const sc_lbm_tuning start = h->tune;
+  const bool given = h->shape_given;
+  // a handle that keeps its default shape keeps the default's rules (no graphs
+  // under an inflow series) with it
+  auto adopt = [&](const sc_lbm_tuning& t) {
+    const int rc = sc_lbm_set_tuning(h, &t);
+    h->shape_given = given || memcmp(&t, &start, sizeof t) != 0;
+    return rc;
+  };
   auto cache = read_cache(cache_path);
   auto it = cache.find(key);
   if (it != cache.end() && it->second.size() == 7) {
     sc_lbm_tuning t{it->second[0], it->second[1], it->second[2], it->second[3],
                     it->second[4], it->second[5], it->second[6]};
-    if (check_tuning(t) == SC_OK) return sc_lbm_set_tuning(h, &t);
+    if (check_tuning(t) == SC_OK) return adopt(t);
   }
   int maxnx = 0;
   for (int d = 0; d < h->P.n_domains; ++d) maxnx = std::max(maxnx, h->P.dom[d].nx);
@@ -1265,7 +1274,7 @@ int sc_lbm_autotune(sc_lbm_t h, const char* cache_path) {
   for (int d = 0; d < h->P.n_domains; ++d) lups += h->P.dom[d].ncell * h->P.dom[d].nodes;
   const int reps = (int)std::max<long long>(4, std::min<long long>(40, 2000000000LL / std::max(1LL, lups)));
   float best = 1e30f;
-  sc_lbm_tuning best_t = h->tune;
+  sc_lbm_tuning best_t = start;
   auto time_it = [&](const sc_lbm_tuning& t, float* ms) -> int {
     int rc = sc_lbm_set_tuning(h, &t);
     if (rc) return rc;
@@ -1327,10 +1336,12 @@ int sc_lbm_autotune(sc_lbm_t h, const char* cache_path) {
     for (int order = 0; order < 2; ++order) cand.push_back({128, 2, 1, order, SC_EXEC_LAUNCH, 50, 1});
   rc = try_all(cand);
   if (rc) { cudaEventDestroy(e0); cudaEventDestroy(e1); return rc; }
-  // execution mode for the best shape
+  // execution mode for the best shape; graphs of as many levels as the handle's
+  // own, where it came with graphs (calls of fewer levels replay none)
   for (int mode : {SC_EXEC_GRAPH, SC_EXEC_PERSISTENT}) {
     sc_lbm_tuning t = best_t;
     t.exec_mode = mode;
+    if (start.exec_mode == SC_EXEC_GRAPH) t.graph_steps = start.graph_steps;
     if (mode == SC_EXEC_PERSISTENT && t.variant == 1) {
       t.variant = 0;  // the persistent form loads one cell per thread
       t.block_x = 64;
@@ -1341,9 +1352,14 @@ int sc_lbm_autotune(sc_lbm_t h, const char* cache_path) {
     if (rc) { cudaEventDestroy(e0); cudaEventDestroy(e1); return rc; }
     if (ms < best * 0.98f) { best = ms; best_t = t; }
   }
+  // the shape and mode the handle came with, which the stages above need not
+  // hold (those of the smallest ensembles are outside them), stay unless
+  // something was faster
+  rc = try_all({start});
+  if (rc) { cudaEventDestroy(e0); cudaEventDestroy(e1); return rc; }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  rc = sc_lbm_set_tuning(h, &best_t);
+  rc = adopt(best_t);
   if (rc) return rc;
   rc = reset_state(h);
   if (rc) return rc;

@@ -131,3 +131,33 @@ def test_while_the_caller_records_another_stream(want):
     assert float(x[0]) == 2.0
     assert np.array_equal(h.state(), want)
     h.close()
+
+
+@pytest.mark.parametrize("size", [(45, 21, 14), (64, 40, 24)])
+def test_autotuned_is_no_slower_than_the_default(size):
+    """Calls of 25 levels, the best of twenty timings before and after: within
+    15% (a tuner without the default among its candidates returned shapes that
+    took 25 and 30% longer)."""
+    import time
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    wl = dict(WL, domains=[dict(WL["domains"][0], nx=size[0], ny=size[1], nz=size[2])])
+    ens = S.Ensemble(S.make_config(wl))
+
+    def best():
+        ens.step(25)
+        ens.sync()
+        out = 1.0
+        for _ in range(20):
+            t = time.perf_counter()
+            for _ in range(10):
+                ens.step(25)
+            ens.sync()
+            out = min(out, time.perf_counter() - t)
+        return out
+
+    default = best()
+    S.sc_lbm_autotune(ens.h, None)
+    tuned = best()
+    assert tuned <= 1.15 * default, (tuned, default, S.sc_lbm_get_tuning(ens.h))
+    ens.close()
