@@ -1632,7 +1632,7 @@ int adj_plan(sc_lbm_t h, int domain, int n_steps, int n_snapshots, int n_probes,
   A.states = off;
   A.K = K;
   A.L = L;
-  A.total = off + A.state_bytes * (size_t)(K + L + 4);
+  A.total = off + A.state_bytes * (size_t)(K + L + 3);  // checkpoints, a segment's later states, 2 forward, 2 adjoint
   return SC_OK;
 }
 }  // namespace
@@ -1706,11 +1706,11 @@ int sc_lbm_adjoint(sc_lbm_t h, int domain, int node, const int32_t* probes, int 
   A.accum = (double*)(ws + L.accum);
   auto state = [&](int k) { return (float*)(ws + L.states + L.state_bytes * (size_t)k); };
   float* snap0 = state(0);           // K checkpoints
-  float* seg0 = state(L.K);          // L segment states
-  float* lamA = state(L.K + L.L);
-  float* lamB = state(L.K + L.L + 1);
-  float* fa = state(L.K + L.L + 2);
-  float* fb = state(L.K + L.L + 3);
+  float* seg1 = state(L.K);          // states 1 .. L - 1 of a segment (its first is the checkpoint)
+  float* lamA = state(L.K + L.L - 1);
+  float* lamB = state(L.K + L.L);
+  float* fa = state(L.K + L.L + 1);
+  float* fb = state(L.K + L.L + 2);
   const long long nstate = (long long)kQ * D.pitch;
   const StepParams& P = h->P;
   auto ck = [&](int r, const char* what) { return r ? cuda_fail(h, (cudaError_t)r, what) : SC_OK; };
@@ -1726,7 +1726,7 @@ int sc_lbm_adjoint(sc_lbm_t h, int domain, int node, const int32_t* probes, int 
   auto issue = [&]() -> int {
     int r;
     auto snap = [&](int k) { return snap0 + (size_t)k * sf; };
-    auto seg = [&](int k) { return seg0 + (size_t)k * sf; };
+    auto seg = [&](int k) { return seg1 + (size_t)(k - 1) * sf; };
     auto forward = [&](const float* src, float* dst, int n) {
       return ck(launch_adj_forward(P, A, src, dst, (float)hn_ramp(h->cfg.ramp_steps, n + 1), h->stream),
                 "adjoint forward");
