@@ -97,8 +97,10 @@ __device__ __forceinline__ void macro(const T g[kQ], T& rho, T& ux, T& uy, T& uz
   rho = SHIFT ? T(1) + m0 : m0;
   if constexpr (sizeof(T) == 4) {
     // one bound for the density and the momentum: with it the quotients stay
-    // below 1e36, and a momentum that is infinite divides
-    if (rho > 1e-18f && (fabsf(jx) + fabsf(jy)) + (fabsf(jz) + rho) < 1e18f) {
+    // below 1e36, and a momentum that is infinite divides (maxima: summed
+    // magnitudes cost the 10-term moments of an odd level 4%, 667 -> 692 us on 25
+    // samples of 160 x 96 x 40)
+    if (rho > 1e-18f && fmaxf(fmaxf(fabsf(jx), fabsf(jy)), fmaxf(fabsf(jz), rho)) < 1e18f) {
       const float r = recip(rho);
       ux = quotient(jx, rho, r);
       uy = quotient(jy, rho, r);
