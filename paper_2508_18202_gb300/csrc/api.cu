@@ -1354,8 +1354,9 @@ int sc_lbm_autotune(sc_lbm_t h, const char* cache_path) {
   }
   // the shape and mode the handle came with, which the stages above need not
   // hold (those of the smallest ensembles are outside them), stay unless
-  // something was faster
-  rc = try_all({start});
+  // something was faster; timed twice, as one interrupted timing of the shortest
+  // levels would lose it
+  rc = try_all({start, start});
   if (rc) { cudaEventDestroy(e0); cudaEventDestroy(e1); return rc; }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
