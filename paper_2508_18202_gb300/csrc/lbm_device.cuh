@@ -222,51 +222,47 @@ __device__ __forceinline__ void all_sums(const T g[kQ], T& m0, T& jx, T& jy, T& 
 // level, launch shape, precision of storage and execution mode, and the
 // adjoint's forward) gives the same bits however the compiler schedules it.
 __device__ __forceinline__ float mul1(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul1(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float add1(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double add1(double a, double b) { return __dadd_rn(a, b); }
 __device__ __forceinline__ float fma1(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma1(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-// BGK with the Smagorinsky effective relaxation time (Sec. 2.2).  SHIFT:
-// populations are g = f - w.  The non-equilibrium stress uses the exact
+// BGK with the Smagorinsky effective relaxation time (Sec. 2.2) on the
+// shifted populations g = f - w.  The non-equilibrium stress uses the exact
 // second moment of the D3Q19 second-order equilibrium, rho/3 I + rho u u.
-template <class T, bool SHIFT>
-__device__ __forceinline__ void collide(T g[kQ], T tau0, T omega0, T smag18c2, bool smag_on) {
-  T m0, jx, jy, jz, pxx, pyy, pzz, pxy, pxz, pyz;
-  all_sums<T>(g, m0, jx, jy, jz, pxx, pyy, pzz, pxy, pxz, pyz);
-  const T rho = SHIFT ? add1(T(1), m0) : m0;
-  const T inv = recip(rho);
-  const T ux = mul1(jx, inv), uy = mul1(jy, inv), uz = mul1(jz, inv);
-  const T usq = fma1(uz, uz, fma1(ux, ux, mul1(uy, uy)));
-  T omega = omega0;
+__device__ __forceinline__ void collide(float g[kQ], float tau0, float omega0, float smag18c2, bool smag_on) {
+  float m0, jx, jy, jz, pxx, pyy, pzz, pxy, pxz, pyz;
+  all_sums<float>(g, m0, jx, jy, jz, pxx, pyy, pzz, pxy, pxz, pyz);
+  const float rho = add1(1.0f, m0);
+  const float inv = recip(rho);
+  const float ux = mul1(jx, inv), uy = mul1(jy, inv), uz = mul1(jz, inv);
+  const float usq = fma1(uz, uz, fma1(ux, ux, mul1(uy, uy)));
+  float omega = omega0;
   if (smag_on) {
-    // Pi^neq = sum c c g - (m0/3 I + rho u u); m0 = rho - 1 (shifted) or rho
-    const T rx = mul1(rho, ux), ry = mul1(rho, uy), rz = mul1(rho, uz);
-    const T nxx = fma1(-rx, ux, fma1(-m0, T(1.0 / 3.0), pxx));
-    const T nyy = fma1(-ry, uy, fma1(-m0, T(1.0 / 3.0), pyy));
-    const T nzz = fma1(-rz, uz, fma1(-m0, T(1.0 / 3.0), pzz));
-    const T nxy = fma1(-rx, uy, pxy);
-    const T nxz = fma1(-rx, uz, pxz);
-    const T nyz = fma1(-ry, uz, pyz);
-    const T dia = fma1(nzz, nzz, fma1(nxx, nxx, mul1(nyy, nyy)));
-    const T off = fma1(nyz, nyz, fma1(nxy, nxy, mul1(nxz, nxz)));
-    const T pin = sqrt(fma1(T(2), fma1(T(2), off, dia), T(1e-30)));
-    omega = recip(mul1(T(0.5), add1(tau0, sqrt(fma1(tau0, tau0, mul1(mul1(smag18c2, pin), inv))))));
+    // Pi^neq = sum c c g - (m0/3 I + rho u u); m0 = rho - 1
+    const float rx = mul1(rho, ux), ry = mul1(rho, uy), rz = mul1(rho, uz);
+    const float nxx = fma1(-rx, ux, fma1(-m0, (float)(1.0 / 3.0), pxx));
+    const float nyy = fma1(-ry, uy, fma1(-m0, (float)(1.0 / 3.0), pyy));
+    const float nzz = fma1(-rz, uz, fma1(-m0, (float)(1.0 / 3.0), pzz));
+    const float nxy = fma1(-rx, uy, pxy);
+    const float nxz = fma1(-rx, uz, pxz);
+    const float nyz = fma1(-ry, uz, pyz);
+    const float dia = fma1(nzz, nzz, fma1(nxx, nxx, mul1(nyy, nyy)));
+    const float off = fma1(nyz, nyz, fma1(nxy, nxy, mul1(nxz, nxz)));
+    const float pin = sqrt(fma1(2.0f, fma1(2.0f, off, dia), 1e-30f));
+    omega = recip(mul1(0.5f, add1(tau0, sqrt(fma1(tau0, tau0, mul1(mul1(smag18c2, pin), inv))))));
   }
   // Opposite pairs (i, i + 1), i odd, share c_i . u up to the sign: the
   // bracket of the equilibrium splits into an even part
-  // m0 + rho (4.5 cu^2 - 1.5 u^2) (m0: w (rho - 1) shifted, w rho plain) and
-  // an odd part 3 rho cu; the weight multiplies last (a rounded 3 w would
-  // bias the momentum of every collision).
-  const T r15 = mul1(T(1.5), usq), r3 = mul1(T(3), rho);
-  g[0] = fma1(-omega, fma1(-W<T>(0), fma1(-rho, r15, m0), g[0]), g[0]);
+  // m0 + rho (4.5 cu^2 - 1.5 u^2) and an odd part 3 rho cu; the weight
+  // multiplies last (a rounded 3 w would bias the momentum of every collision).
+  const float r15 = mul1(1.5f, usq), r3 = mul1(3.0f, rho);
+  g[0] = fma1(-omega, fma1(-W<float>(0), fma1(-rho, r15, m0), g[0]), g[0]);
 #pragma unroll
   for (int i = 1; i < kQ; i += 2) {
-    const T cu = cdot<T>(i, ux, uy, uz);
-    const T even = fma1(rho, fma1(mul1(T(4.5), cu), cu, -r15), m0);
-    g[i] = fma1(-omega, fma1(-W<T>(i), fma1(r3, cu, even), g[i]), g[i]);
-    g[i + 1] = fma1(-omega, fma1(-W<T>(i), fma1(-r3, cu, even), g[i + 1]), g[i + 1]);
+    const float cu = cdot<float>(i, ux, uy, uz);
+    const float even = fma1(rho, fma1(mul1(4.5f, cu), cu, -r15), m0);
+    g[i] = fma1(-omega, fma1(-W<float>(i), fma1(r3, cu, even), g[i]), g[i]);
+    g[i + 1] = fma1(-omega, fma1(-W<float>(i), fma1(-r3, cu, even), g[i + 1]), g[i + 1]);
   }
 }
 
@@ -400,7 +396,7 @@ __device__ __forceinline__ void collide_rr(T g[kQ], T tau0, T smag18c2, bool sma
 }
 
 // ------------------------------------------------------------ two cells at once
-// The BGK(+Smagorinsky) collision of collide<float, true> for two cells, one
+// The BGK(+Smagorinsky) collision of collide() for two cells, one
 // in each lane of Blackwell's packed FP32x2 operations (__fadd2_rn,
 // __fmul2_rn, __ffma2_rn; each lane rounds as the scalar operation does):
 // the even level of the 16-bit storage modes, at half the arithmetic
@@ -538,7 +534,7 @@ __device__ __forceinline__ void collide_p(const StepParams& P, T g[kQ]) {
   if constexpr (sizeof(T) == 8)
     collide_fp64(g, P.tau0_d, P.omega0_d, P.smag18c2_d, P.csmag_on);
   else
-    collide<T, SHIFT>(g, T(P.tau0), T(P.omega0), T(P.smag18c2), P.csmag_on);
+    collide(g, P.tau0, P.omega0, P.smag18c2, P.csmag_on);
 #endif
 }
 

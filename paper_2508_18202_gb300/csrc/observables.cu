@@ -639,7 +639,8 @@ __global__ void export_kernel(const __grid_constant__ StepParams P, int domain, 
 // Sec. 2.4 step 6): adds |u| at the current level, per (node, cell), in FP64.
 // One cell a thread, gridDim.y over the nodes (64-bit divisions of one long
 // index were half of the kernel's instructions).  13 samples of 192 x 96 x 64,
-// odd level: 485 -> 343 us (even 235 -> 205, of a floor of 207).
+// odd level: 485 -> 343 us (even 235 -> 205; the 92 bytes of each fluid cell take
+// 193 at the copy rate).
 template <class S, bool SHIFT, bool ODD>
 __global__ void __launch_bounds__(256) average_add_kernel(const __grid_constant__ StepParams P, int domain, double* avg) {
   using T = typename Store<S>::C;
@@ -868,6 +869,8 @@ int launch_moments(const StepParams& P, int precision, const MomentArgs& A, void
     if (A.mean) {
       const unsigned grid = (unsigned)((D.ncell + blk - 1) / blk);
       if (A.P > kMaxGpcP) return (int)cudaErrorInvalidValue;
+      // averages are scaled after their sums, with any value those start from
+      if (A.avg && A.accumulate) return (int)cudaErrorInvalidValue;
       auto pair = [&](auto pm) {
         constexpr int PM = decltype(pm)::value;
         if constexpr (SH && PM <= kMomCellMaxP) {
