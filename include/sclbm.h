@@ -187,7 +187,7 @@ typedef struct {
  * equal the one-cell form's to FP32 rounding, not bit for bit.  Default:
  * tile order 1, variant 0, block, slab and mode (launch, or graph for the
  * smallest ensembles) by the ensemble's size and collision; sc_lbm_get_tuning
- * names them.                                                               */
+ * names them.  The FP64 path has one shape of its own and ignores these.     */
 typedef struct {
   int block_x, block_y, slab_z, tile_order, exec_mode, graph_steps, variant;
 } sc_lbm_tuning;

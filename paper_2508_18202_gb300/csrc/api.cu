@@ -411,14 +411,27 @@ void apply_tiling(sc_lbm_t h) {
 
 // The launch shape of a handle that is neither tuned nor given one.  Rows of
 // 32 cells waste the least on a width that is no multiple of the block, and
-// blocks of two rows leave the level's last wave short.  Even + odd level in us
-// against 64 x 2 x 8, BGK: 13 samples of 256 x 128 x 64 FP32 1357 -> 1310 at
-// 32 x 2 x 4, 3 of 512 x 256 x 128 2543 -> 2466, 13 of 97 x 61 x 33 164 -> 154
-// (32 x 2 x 2: 151), FP16 131 -> 127.  A thread walks its slab serially, so a
-// level that leaves the chip idle takes shorter ones: 13 of 64 x 40 x 24 59 -> 51
-// at 32 x 2 x 2 (4: 55), 3 of 45 x 21 x 14 28.7 -> 16.4 at 32 x 1 x 1 (32 x 2 x 2: 16.9).
-// The regularized collision carries more arithmetic per cell and gains from
-// longer slabs: 25 of 120 x 120 x 40 787 -> 762 at 32 x 4 x 8 (32 x 2 x 4: 771).
+// blocks of two rows leave the level's last wave short; a thread walks its slab
+// serially, so a level that leaves the chip idle takes shorter ones.  us a level
+// (mean of even and odd), the class's shape / 64 x 2 x 8 in launches:
+//   samples             BGK FP32       BGK BF16       RR FP32        RR BF16
+//   below 0.2 M cells: 32 x 1 x 1, graphs of eight levels
+//   3 of 45 x 21 x 14    4.4 / 12.0     4.9 / 12.4     5.4 / 15.4     5.7 / 15.4
+//   5 of 48 x 24 x 24    8.2 / 13.7     7.7 / 16.5     9.1 / 17.5     9.5 / 17.5
+//   below 4 M: 32 x 2 x 2
+//   9 of 48 x 48 x 14   13.7 / 16.5    16.3 / 19.5    16.6 / 20.7    17.6 / 21.3
+//   9 of 97 x 61 x 33   52.1 / 56.7    45.1 / 48.3    59.7 / 64.1    58.2 / 61.1
+//   4 of 96 x 96 x 96   98.4 / 103.8   80.2 / 83.5   109.0 / 114.1  101.5 / 104.5
+//   from 4 M on: 32 x 2 x 4, the regularized collision 32 x 4 x 8
+//   4 of 192 x 96 x 64  122.9 / 128.6  89.9 / 96.2   135.8 / 136.4  121.8 / 122.5
+//   25 of 65 x 129 x 31 187.3 / 194.7 157.0 / 152.4  207.1 / 208.2  186.9 / 189.8
+//   25 of 120 x 120 x 40 384.7 / 410.3 284.0 / 291.7 426.5 / 428.7  376.3 / 377.3
+//   9 of 256 x 128 x 64 458.7 / 478.7 319.0 / 323.4  496.1 / 497.7  435.9 / 437.1
+// Next to the lines: 32 x 2 x 2 in launches takes 9.7 at 5 of 48 x 24 x 24 FP32, and
+// slabs of 2 and 4 are even at 4 of 96 x 96 x 96 (98.4, 97.9).  The longer slabs of
+// the regularized collision, which carries more arithmetic per cell, pay in 16
+// bits (25 of 120 x 120 x 40: 376.3, 388.7 at 32 x 2 x 4) and on large FP32 nodes (9
+// of 192 x 96 x 64: 286.1, 288.4), not on small ones (25 of 120 x 120 x 40: 426.5, 416.2).
 sc_lbm_tuning default_tuning(const sc_lbm_t h) {
   sc_lbm_tuning t;
   t.variant = 0;

@@ -19,7 +19,8 @@
 // Bound: latency of a block's passes over its values (16 warps an SM, the
 // shared memory holds 8 cells' values).  4096 cells, 4096 samples, 21 terms: a
 // bitonic sort of the FP64 values of each cell took 4848 us (FP64 compares,
-// pipe 82% busy), this form takes 152 us.
+// pipe 82% busy), this form takes 152 us.  Where every cell is sorted whole the
+// call takes 2.17 ms (5.10 with that sort alone; 1000 samples: 0.64 and 1.04).
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -31,6 +32,7 @@ namespace sclbm {
 namespace {
 
 constexpr int kThreads = 512;
+constexpr int kSMs = 152;
 constexpr int kBuckets = 1024;
 constexpr int kCandidates = 192;  // exact evaluations held per (cell, quantile)
 
@@ -311,9 +313,9 @@ int launch_gpc_quantiles(const double* coef, long long ncell, int P, const int32
   // eight cells share a basis value while their FP32 values fit the shared
   // memory of one block an SM (and the cells fill the chip); four above 4096
   // samples; one when there are few cells
-  if (n_cells < 152 * 2)
+  if (n_cells < 2 * kSMs)
     return launch_group<1>(coef, ncell, P, cells, n_cells, phi, phif, M, Mf, Mp, bound, kidx, nq, out, s);
-  if (M > 4096 || n_cells < 152 * 8)
+  if (M > 4096 || n_cells < 8 * kSMs)
     return launch_group<4>(coef, ncell, P, cells, n_cells, phi, phif, M, Mf, Mp, bound, kidx, nq, out, s);
   return launch_group<8>(coef, ncell, P, cells, n_cells, phi, phif, M, Mf, Mp, bound, kidx, nq, out, s);
 }
