@@ -562,13 +562,15 @@ struct Node {
 
 // 6 w_i (c_i . u) r, direction i known at compile time; u is the wall
 // velocity turned to the arrival level's direction, r its scale.
-template <class T>
+// FULL: c_i . u with its products by zero (the same value).
+template <class T, bool FULL = false>
 __device__ __forceinline__ T wall_term(int i, T ux, T uy, T uz, T r) {
-  return T(6) * W<T>(i) * cdot<T>(i, ux, uy, uz) * r;
+  const T cu = FULL ? T(CX(i)) * ux + T(CY(i)) * uy + T(CZ(i)) * uz : cdot<T>(i, ux, uy, uz);
+  return T(6) * W<T>(i) * cu * r;
 }
 
 // Pull of the odd AA level (swapped layout in place).
-template <class S, bool CG>
+template <class S, bool CG, bool FULL = false>
 __device__ __forceinline__ void fast_pull(const S* base, LinkWord lw, int pc, int sy, int sz,
                                           typename Store<S>::C ux, typename Store<S>::C uy,
                                           typename Store<S>::C uz, typename Store<S>::C r,
@@ -581,7 +583,7 @@ __device__ __forceinline__ void fast_pull(const S* base, LinkWord lw, int pc, in
     const int spec = OPP(REFL(i, 2)) * pc - (CX(i) + CY(i) * sy);
     const int off = kind == kStream ? stream : (kind == kSpecZ ? spec : i * pc);
     T v = LD<S, CG>(base + off);
-    if (kind == kMoving) v += wall_term<T>(i, ux, uy, uz, r);
+    if (kind == kMoving) v += wall_term<T, FULL>(i, ux, uy, uz, r);
     g[i] = v;
   }
 }
@@ -692,7 +694,7 @@ __device__ __forceinline__ ListedRef listed_ref(const DevDomain& D, long long li
 
 // Pull of the odd AA level for a listed cell from its compiled rules: g0 is
 // the node's population base, bo its outflow plane (float).
-template <class S, bool CG>
+template <class S, bool CG, bool FULL = false>
 __device__ __forceinline__ void listed_pull(const ListedRef& L, const S* g0, const float* bo,
                                             typename Store<S>::C ux, typename Store<S>::C uy,
                                             typename Store<S>::C uz, typename Store<S>::C r,
@@ -703,7 +705,7 @@ __device__ __forceinline__ void listed_pull(const ListedRef& L, const S* g0, con
   for (int i = 0; i < kQ; ++i) {
     const int s = L.word(kWordSrc + i);
     T v = ((bm >> i) & 1u) ? T(__ldcg(bo + s)) : LD<S, CG>(g0 + s);
-    if ((pm >> i) & 1u) v += wall_term<T>(i, ux, uy, uz, r);
+    if ((pm >> i) & 1u) v += wall_term<T, FULL>(i, ux, uy, uz, r);
     g[i] = v;
   }
 }

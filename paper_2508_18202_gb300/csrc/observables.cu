@@ -59,16 +59,21 @@ __device__ __forceinline__ void gather_pops(const StepParams& P, const DevDomain
 #pragma unroll
       for (int i = 0; i < kQ; ++i) g[i] = Store<S>::ld(N.g + (long long)i * D.pitch + idx);
     } else {
-      // P.wp is the inflow factor of level n (the launch's n_host)
+      // P.wp is the inflow factor of level n (the launch's n_host).  FP32 storage
+      // takes the wall terms with their products by zero: without them the
+      // exported velocity of an odd level reads 83 us on 256 x 128 x 64 and 51 on
+      // 192 x 96 x 64, with them 73 and 45 (on 384 x 160 x 72 136 and 138); in 16 bits
+      // 85 and 86, 45 and 47, 148 and 160.
+      constexpr bool FULL = sizeof(S) == 4;
       T ux, uy, uz;
       if (lw & kLinkSlow) {
         const ListedRef L = listed_ref(D, listed_index(D, idx));
         inflow_velocity<S>(N, z, wind_pull<T>(P), ux, uy, uz);
-        listed_pull<S, false>(L, N.g, N.bout, ux, uy, uz, wind_pull<T>(P).scale, g);
+        listed_pull<S, false, FULL>(L, N.g, N.bout, ux, uy, uz, wind_pull<T>(P).scale, g);
       } else {
         wall_velocity<S>(N, lw, z, wind_pull<T>(P), ux, uy, uz);
-        fast_pull<S, false>(N.g + idx, lw, (int)D.pitch, D.nx, D.nx * D.ny, ux, uy, uz, wind_pull<T>(P).scale,
-                            g);
+        fast_pull<S, false, FULL>(N.g + idx, lw, (int)D.pitch, D.nx, D.nx * D.ny, ux, uy, uz,
+                                  wind_pull<T>(P).scale, g);
       }
     }
   }
