@@ -369,7 +369,10 @@ __device__ __forceinline__ void with_pops_form(LinkWord lw, F&& f) {
 // too many accumulators per thread for it and goes to moments_split_kernel.
 // Up to 10 terms three blocks are resident per SM (80 registers); four at 10
 // terms and an even level, which holds no links (2.43 -> 2.30 ms on 6 samples of
-// 512 x 256 x 128; no gain below).
+// 512 x 256 x 128; no gain below).  At an odd level the 80 registers spill: 8 to
+// 56 bytes up to 8 terms, 136 to 148 at 10, where two blocks without spills are
+// slower in FP32 and faster in 16 bits (25 samples of 160 x 96 x 40, three / two
+// blocks: FP32 668 / 677 us, BF16 624 / 563).
 // Bound: the FP64 pipe where the nodes are few (16 cycles of an SM for an
 // instruction of a warp), so conversions go by the bits, the sums are only
 // converted where they continue, and a mean divides by a reciprocal; else the
